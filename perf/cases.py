@@ -162,11 +162,12 @@ def _mlp(case, seed):
 
     site = unit(0.5 + 0.1 * normal(n, 2 * D ** 4))
     eye = torch.eye(D, device="cuda", dtype=torch.float64)
-    root = eye + 0.3 * normal(n, D, D)
-    sig = unit(root @ root.mT)
-    low = torch.linalg.cholesky(sig + 1e-12 * eye)
+    low = torch.tril(0.3 * normal(n, D, D), -1) + eye * (1.0 + 0.3 * normal(n, D, 1).clamp(-2.0, 2.0))
+    sig = low @ low.mT
+    size = sig.square().sum(dim=(1, 2), keepdim=True).sqrt()
+    sig, low = sig / size, low / size.sqrt()
     X = torch.cat([site, sig.reshape(n, -1), low.reshape(n, -1)], dim=1).float().contiguous()
-    near = root + 0.05 * normal(n, D, D)
+    near = low + 0.05 * normal(n, D, D)
     Y = unit(near @ near.mT).reshape(n, -1).float().contiguous()
     w = peps.mlp_init(2, D, seed=seed)
     # a network that has been trained for a while: the output layer is no longer zero
