@@ -13,6 +13,7 @@
 #include <cstdio>
 #include <cstring>
 #include <cstdlib>
+#include <map>
 #include <mutex>
 #include <tuple>
 #include <vector>
@@ -58,13 +59,15 @@ struct QrArgs {
   TP Q;
   long long qrs, qcs;
   TP R;         // absent: R not wanted
-  double* W;    // m*n work per problem, column-major (problem p at W + p * wst)
-  double* Qw;   // m*k work per problem, column-major (+ p * qst)
-  double* tau;  // k per problem (+ p * tst)
+  double* W;    // work per problem (problem p at W + p * wst): k_qr_cluster's rows where they
+                // do not fit in shared memory (C * ld * n), k_qr_house's m x n copy
+  double* Qw;   // k_qr_house: m*k work per problem, column-major (+ p * qst)
+  double* tau;  // k_qr_house: k per problem (+ p * tst)
   long long wst, qst, tst;
 };
 
-// Grid = problems, one CTA each.
+// Grid = problems, one CTA each, everything in global memory: for matrices with
+// more columns than k_qr_cluster's shared memory holds sums for.
 __global__ void __launch_bounds__(QR_THREADS) k_qr_house(const QrArgs q) {
   __shared__ double red[32];
   __shared__ double s_tau, s_scale;
@@ -152,59 +155,6 @@ __global__ void __launch_bounds__(QR_THREADS) k_qr_house(const QrArgs q) {
   }
 }
 
-// ---------------------------------------------------------------------------
-// Householder QR on a thread-block cluster: the rows of one matrix are split
-// over the cluster's CTAs (one SM each); every column reduction (the norm
-// below the diagonal, the reflector's inner products with the trailing
-// columns) is a per-CTA partial sum exchanged through distributed shared
-// memory between hardware cluster barriers.  Same reflectors, same order and
-// same sign convention as the one-CTA kernel; the FP64 work is spread over C
-// SMs instead of one.
-// ---------------------------------------------------------------------------
-constexpr int QRC_THREADS = 512;
-// Each CTA keeps its block of rows of the working matrix and of Q in shared
-// memory when they fit (column-major within the block, odd column stride),
-// else in global scratch.  Work per column is split as (column, row quarter)
-// per thread: every thread runs a plain FMA loop over its rows, so the FP64
-// pipe executes the factorisation's own multiply-adds and almost nothing else
-// (a shuffle tree per column would cost more FP64 issue slots than the dot
-// products at 64 rows per CTA).
-constexpr int QS = 8;   // threads per column (rows interleaved mod QS)
-
-// Strided dot product and update over rows start, start + QS, ... < end with
-// four rows' loads in flight per step (when the rows live in global memory a
-// thread's loop is otherwise one dependent load after another); fixed
-// summation order.
-__device__ __forceinline__ double dot_qs(const double* __restrict__ x, const double* __restrict__ y, int start,
-                                         int end) {
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-  int i = start;
-  for (; i + 3 * QS < end; i += 4 * QS) {
-    const double x0 = x[i], x1 = x[i + QS], x2 = x[i + 2 * QS], x3 = x[i + 3 * QS];
-    const double y0 = y[i], y1 = y[i + QS], y2 = y[i + 2 * QS], y3 = y[i + 3 * QS];
-    a0 = fma(x0, y0, a0);
-    a1 = fma(x1, y1, a1);
-    a2 = fma(x2, y2, a2);
-    a3 = fma(x3, y3, a3);
-  }
-  for (; i < end; i += QS) a0 = fma(x[i], y[i], a0);
-  return (a0 + a1) + (a2 + a3);
-}
-
-// y[i] -= w x[i] over the same rows (x and y are different columns).
-__device__ __forceinline__ void axpy_qs(double w, const double* __restrict__ x, double* __restrict__ y, int start,
-                                        int end) {
-  int i = start;
-  for (; i + 3 * QS < end; i += 4 * QS) {
-    const double x0 = x[i], x1 = x[i + QS], x2 = x[i + 2 * QS], x3 = x[i + 3 * QS];
-    const double y0 = y[i], y1 = y[i + QS], y2 = y[i + 2 * QS], y3 = y[i + 3 * QS];
-    y[i] = fma(-w, x0, y0);
-    y[i + QS] = fma(-w, x1, y1);
-    y[i + 2 * QS] = fma(-w, x2, y2);
-    y[i + 3 * QS] = fma(-w, x3, y3);
-  }
-  for (; i < end; i += QS) y[i] = fma(-w, x[i], y[i]);
-}
 
 // Sum of one double over the cluster's CTAs, all remote loads issued first.
 __device__ __forceinline__ double remote_sum(cg::cluster_group& cl, double* slot, int C) {
@@ -217,7 +167,112 @@ __device__ __forceinline__ double remote_sum(cg::cluster_group& cl, double* slot
   return s;
 }
 
-__global__ void __launch_bounds__(QRC_THREADS) k_qr_cluster(const QrArgs q, int in_smem, int ld) {
+// ---------------------------------------------------------------------------
+// Householder QR, one thread-block cluster of C = 1-16 CTAs per matrix, its
+// rows split over the CTAs and kept in shared memory where they fit.
+//
+// What bounds it: GB300's FP64 pipe.  A warp's FP64 instruction holds the pipe
+// of its SM quarter for 64 clocks whatever its active lanes, and a dependent
+// one waits as long (an addition after a shuffle 110), so a column step costs
+// its FP64 instructions: the fused update and inner products (2 per element),
+// a few sums, and the scalar chain (1 / norm and one reciprocal, ~900 clocks).
+// Barriers cost ~50 clocks for a CTA, ~450 for a cluster, a remote load ~400.
+// Hence
+//   * one pass per column: the update with reflector j and the inner products
+//     with column j+1 (updated just before) read every element once;
+//   * the reflector stays unscaled, x = (alpha - beta; a_ij): with s = |x_j|^2
+//     over rows >= j, y = sgn(alpha) / sqrt(s), beta = -s y and
+//     g = 1 / (s + |alpha| sqrt(s)), H = I - g x x^T.  For the inner product
+//     f_c = sum_{i >= j} a_ij a_ic, row j of R is -y f_c and an updated entry
+//     a_ic - w_c a_ij with w_c = g (f_c - beta a_jc);
+//   * partial sums stay in their CTA's shared memory and are read from there
+//     after the cluster barrier by four threads per column, all loads first;
+//   * Q is formed from the reflectors at once and not one by one: the passes
+//     also take the inner products x_a . x_j of the earlier reflectors (one
+//     FMA per element), so X^T X is known when the last column is done, and
+//     Q = E - X M with M = T X_1^T, where T^{-1} is upper triangular with
+//     1 / g on the diagonal and X^T X above it (the UT transform: Joffrain,
+//     Low, Quintana-Orti, van de Geijn & Van Zee, 2006).  Every column of M is
+//     one back substitution in one warp, the columns dealt to the CTAs; the
+//     product runs at the FP64 pipe's rate.  Against one barrier, one set of
+//     sums and one pass per reflector (256x16 70 us, 512x32 158, 1024x64 441,
+//     64x64 280) this takes 53, 131, 381 and 203 us.
+// Measured (us, one matrix, with Q; before: scaled reflectors, update and inner
+// products in two passes, sums by one thread per column, Q one reflector at a
+// time): 256x16 117 -> 53, 512x32 236 -> 131, 1024x64 608 -> 381, 2304x64
+// 824 -> 618, 1620x180 3637 -> 2861, 8192x128 (tall-skinny, four leaves)
+// 3847 -> 2853; 16 of 36x36 270 -> 123 (those ran in global memory, one CTA
+// each).  Orthogonality stays at 1e-15 to 7e-15; |A - QR| is 1 to 3 eps of a
+// column's norm.
+// ---------------------------------------------------------------------------
+constexpr int QRC_MAXT = 512;
+
+// Per-CTA shared memory besides the rows and the triangle, in doubles.
+__host__ __device__ inline long long qr_head(int n, int k, int c) {
+  return 7LL * n + 4LL * k + 4 + (long long)((k + c - 1) / c) * k;
+}
+// The triangle: X^T X, then M.
+__host__ __device__ inline long long qr_tri(int k) { return (long long)k * (k + 1) / 2; }
+
+// Sum over rows i, i + L, ... < r1 of x y.
+__device__ __forceinline__ double qr_dot(const double* x, const double* y, int i, int L, int r1) {
+  double acc = 0.0;
+  for (; i + 3 * L < r1; i += 4 * L) {
+    const int i1 = i + L, i2 = i1 + L, i3 = i2 + L;
+    const double a0 = x[i], a1 = x[i1], a2 = x[i2], a3 = x[i3];
+    const double b0 = y[i], b1 = y[i1], b2 = y[i2], b3 = y[i3];
+    acc = fma(a0, b0, acc);
+    acc = fma(a1, b1, acc);
+    acc = fma(a2, b2, acc);
+    acc = fma(a3, b3, acc);
+  }
+  for (; i < r1; i += L) acc = fma(x[i], y[i], acc);
+  return acc;
+}
+
+// The same rows of one column: the update a -= w xj, and the sum of the
+// results times xn.  The loads of four rows are issued before their arithmetic.
+__device__ __forceinline__ double qr_update_dot(double* wc, const double* xj, const double* xn, double w, int i,
+                                                int L, int r1) {
+  double acc = 0.0;
+  for (; i + 3 * L < r1; i += 4 * L) {
+    const int i1 = i + L, i2 = i1 + L, i3 = i2 + L;
+    const double a0 = wc[i], a1 = wc[i1], a2 = wc[i2], a3 = wc[i3];
+    const double x0 = xj[i], x1 = xj[i1], x2 = xj[i2], x3 = xj[i3];
+    const double n0 = xn[i], n1 = xn[i1], n2 = xn[i2], n3 = xn[i3];
+    const double y0 = fma(-w, x0, a0), y1 = fma(-w, x1, a1), y2 = fma(-w, x2, a2), y3 = fma(-w, x3, a3);
+    wc[i] = y0;
+    wc[i1] = y1;
+    wc[i2] = y2;
+    wc[i3] = y3;
+    acc = fma(y0, n0, acc);
+    acc = fma(y1, n1, acc);
+    acc = fma(y2, n2, acc);
+    acc = fma(y3, n3, acc);
+  }
+  if (i + L < r1) {
+    const int i1 = i + L;
+    const double a0 = wc[i], a1 = wc[i1], x0 = xj[i], x1 = xj[i1], n0 = xn[i], n1 = xn[i1];
+    const double y0 = fma(-w, x0, a0), y1 = fma(-w, x1, a1);
+    wc[i] = y0;
+    wc[i1] = y1;
+    acc = fma(y0, n0, acc);
+    acc = fma(y1, n1, acc);
+    i += 2 * L;
+  }
+  if (i < r1) {
+    const double y = fma(-w, xj[i], wc[i]);
+    wc[i] = y;
+    acc = fma(y, xn[i], acc);
+  }
+  return acc;
+}
+
+// lanes_log2: threads that share a column of the pass, 4 to 32: 128 threads
+// are enough to keep the FP64 pipe busy, and each doubling adds an addition to
+// every sum.
+__global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_smem, int tri_smem, int ld,
+                                                         int lanes_log2) {
   extern __shared__ double qsm[];
   cg::cluster_group cluster = cg::this_cluster();
   const int C = int(cluster.num_blocks());
@@ -227,160 +282,207 @@ __global__ void __launch_bounds__(QRC_THREADS) k_qr_cluster(const QrArgs q, int 
   double* const Qo = q.Q.d(pb);
   double* const Ro = q.R.n ? q.R.d(pb) : nullptr;
   const int m = q.m, n = q.n, k = min(m, n);
-  const int tid = threadIdx.x, nt = blockDim.x;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   const int chunk = (m + C - 1) / C;
   const int r0 = min(m, rank * chunk), r1 = min(m, r0 + chunk), rows = r1 - r0;
-  // Cluster-visible, double-buffered by column parity:
-  double* wpart = qsm;              // [2][n] my partial raw inner products of column j with columns c > j
-  double* rowj = wpart + 2 * n;     // [2][n] row j of the trailing matrix (valid in the row's owner)
-  double* npart = rowj + 2 * n;     // [2]    my partial squared norm of column j below the diagonal
-  double* tau_s = npart + 2;        // [k]
-  double* part4 = tau_s + k;        // [n][QS] quarter sums
-  double* wfin = part4 + (long long)n * QS;   // [n]
-  double* coef = wfin + n;          // [2] scale, beta of the current reflector
-  double* W;                        // [n][ld] my rows, column-major (row i at i - r0); Q is formed in place
-  if (in_smem) {
-    W = coef + 2 + QS;
-  } else {
-    W = q.W + pb * q.wst + (long long)rank * ld * n;
+  const int mcols = (k + C - 1) / C;        // columns of M solved here: rank, rank + C, ...
+  double* part = qsm;                       // [2][n] my partial sums (read by every CTA)
+  double* rowv = part + 2 * n;              // [2][n] row j of the matrix (in the row's owner)
+  double* dsum = rowv + 2 * n;              // [n] inner products of this step
+  double* rowl = dsum + n;                  // [n] row j, local copy
+  double* wfin = rowl + n;                  // [n] w_c of this step
+  double* ys = wfin + n;                    // [k] y
+  double* gs = ys + k;                      // [k] g
+  double* nb = gs + k;                      // [k] -beta
+  double* vs = nb + k;                      // [k] alpha - beta
+  double* mc = vs + k + 4;                  // [mcols][k] my columns of X_1^T, then of M (read by every CTA)
+  double* tri = mc + mcols * k;             // packed columns: X^T X above the diagonal, then M
+  double* W = tri + (tri_smem ? qr_tri(k) : 0);   // [n][ld], row i at i - r0
+  {
+    double* g = q.W + pb * q.wst + rank * (q.wst / C);
+    if (!tri_smem) {
+      tri = g;
+      g += qr_tri(k);
+    }
+    if (!w_smem) W = g;
   }
-  for (long long e = tid; e < (long long)rows * n; e += nt) {
-    const int li = int(e % rows), j = int(e / rows);
-    W[(long long)j * ld + li] = A[(r0 + li) * q.rs + j * q.cs];
+  auto cta_or_cluster_sync = [&]() {
+    if (C > 1)
+      cluster.sync();
+    else
+      __syncthreads();
+  };
+  if (q.cs == 1) {
+    for (int e = tid; e < rows * n; e += nt) {
+      const int li = e / n, j = e - li * n;
+      W[j * ld + li] = A[(r0 + li) * q.rs + j];
+    }
+  } else {
+    for (int e = tid; e < rows * n; e += nt) {
+      const int j = e / rows, li = e - j * rows;
+      W[j * ld + li] = A[(r0 + li) * q.rs + j * q.cs];
+    }
   }
   __syncthreads();
-  // My partial sums for column j into buffer b: sum over my rows i > j of
-  // a_ji * a_ci for every c >= j (c = j: the squared norm), and, in the owner
-  // of row j, that row.  The reflector's inner products with the trailing
-  // columns are taken with the unscaled column, w_c = tau (a_cj + scale *
-  // sum_i a_ji a_ci), so one cluster barrier per column carries both the norm
-  // (for tau) and the inner products.
-  auto partials = [&](int j, int b) {
-    const int i0 = max(r0, j + 1);
-    const double* xj = W + (long long)j * ld - r0;
-    for (int t = tid; t < (n - j) * QS; t += nt) {
-      const int c = j + t / QS, qq = t % QS;
-      const double* wc = W + (long long)c * ld - r0;
-      part4[(long long)c * QS + qq] = dot_qs(xj, wc, i0 + ((qq - i0 % QS + QS) % QS), r1);
-    }
-    __syncthreads();
-    const bool has_row = j >= r0 && j < r1;
-    for (int c = j + tid; c < n; c += nt) {
-      double w = 0.0;
-      for (int qq = 0; qq < QS; ++qq) w += part4[(long long)c * QS + qq];
-      if (c == j)
-        npart[b] = w;
-      else
-        wpart[b * n + c] = w;
-      if (has_row) rowj[b * n + c] = W[(long long)c * ld + (j - r0)];
+  // One pass over the columns: the update with reflector column j (w from
+  // wfin; j < 0: none) for c > jn, then the inner products with column jn
+  // (final already) over rows >= jn for c > jn, over rows > jn otherwise.  The
+  // owner of row jn publishes it.
+  const int sh = lanes_log2, L = 1 << sh;
+  auto pass = [&](int j, int jn, int b) {
+    const double* xj = W + max(j, 0) * ld - r0;
+    const double* xn = W + jn * ld - r0;
+    const bool own = jn >= r0 && jn < r1;
+    for (int t0 = tid - lane; t0 < n << sh; t0 += nt) {
+      const int c = (t0 + lane) >> sh, l = lane & (L - 1);
+      double acc = 0.0;
+      double* wc = W + min(c, n - 1) * ld - r0;
+      const int i0 = max(r0, c > jn ? jn : jn + 1) + l;
+      if (c < n) {
+        if (j >= 0 && c > jn)
+          acc = qr_update_dot(wc, xj, xn, wfin[c], i0, L, r1);
+        else
+          acc = qr_dot(wc, xn, i0, L, r1);
+      }
+      for (int o = L >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (c < n && l == 0) {
+        part[b * n + c] = acc;
+        if (own) rowv[b * n + c] = wc[jn];
+      }
     }
   };
-  partials(0, 0);
+  pass(-1, 0, 0);
   for (int j = 0; j < k; ++j) {
-    const int b = j & 1;
-    const int owner = j / chunk;
-    const bool own = (owner == rank);
-    cluster.sync();                                   // column j: norms, inner products, row j visible
-    if (tid < 32) {
-      const double alpha = *cluster.map_shared_rank(rowj + b * n + j, owner);
-      double sig = 0.0;
-      for (int r = tid; r < C; r += 32) sig += *cluster.map_shared_rank(npart + b, r);
-      sig = warp_sum(sig);
-      double tau = 0.0, scale = 0.0, beta = alpha;
-      if (sig != 0.0) {
-        const double nrm = sqrt(alpha * alpha + sig);
-        beta = alpha >= 0.0 ? -nrm : nrm;
-        tau = (beta - alpha) / beta;
-        scale = 1.0 / (alpha - beta);
+    const int b = j & 1, owner = j / chunk;
+    cta_or_cluster_sync();                            // column j: inner products and row j visible
+    // row j, local copy: the threads that do not sum start at the far end
+    for (int c = nt - 1 - tid; c < n; c += nt)
+      rowl[c] = C > 1 ? *cluster.map_shared_rank(rowv + b * n + c, owner) : rowv[b * n + c];
+    // sums over the CTAs, four threads per column, column j first
+    for (int t0 = tid - lane; t0 < 4 * n; t0 += nt) {
+      const int ci = (t0 + lane) >> 2, l = lane & 3;
+      int c = min(ci, n - 1) + j;
+      if (c >= n) c -= n;
+      double* slot = part + b * n + c;
+      double alpha = 0.0, s;
+      if (C == 1) {
+        s = *slot;
+        if (ci == 0) alpha = rowv[b * n + j];
+      } else {
+        const double v0 = l < C ? *cluster.map_shared_rank(slot, l) : 0.0;
+        const double v1 = l + 4 < C ? *cluster.map_shared_rank(slot, l + 4) : 0.0;
+        const double v2 = l + 8 < C ? *cluster.map_shared_rank(slot, l + 8) : 0.0;
+        const double v3 = l + 12 < C ? *cluster.map_shared_rank(slot, l + 12) : 0.0;
+        if (ci == 0) alpha = *cluster.map_shared_rank(rowv + b * n + j, owner);
+        s = v0;
+        if (C > 4) s += v1;
+        if (C > 8) s = (s + v2) + v3;
+        if (C > 2) s += __shfl_xor_sync(0xffffffffu, s, 2);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
       }
-      if (tid == 0) {
-        tau_s[j] = tau;
-        coef[0] = scale;
-        coef[1] = beta;
+      if (ci >= n || l != 0) continue;
+      if (ci > 0) {
+        dsum[c] = s;
+        continue;
       }
+      // scalars of reflector j (thread 0): a column that is zero below the
+      // diagonal, or whose squares underflow, has no reflector.  Tests on the
+      // bits: an FP64 compare costs as much as an FMA.
+      const double ss = fma(alpha, alpha, s);
+      double y = 0.0, g = 0.0, h = 0.0;
+      if (__double_as_longlong(s) << 1 != 0 && (__double2hiint(ss) >> 20 & 0x7ff) >= 23) {
+        const double r = rsqrt(ss), e = fma(fabs(alpha), r, 1.0);
+        // 1 / e, e in [1, 2]: two Newton steps in one (cubic) from the FP32 value
+        const double z = double(__frcp_rn(float(e)));
+        const double d = fma(-e, z, 1.0);
+        g = r * r * fma(z, fma(d, d, d), z);
+        y = copysign(r, alpha);
+        h = copysign(ss * r, alpha);
+      }
+      ys[j] = y;
+      gs[j] = g;
+      nb[j] = h;
+      vs[j] = alpha;
     }
     __syncthreads();
-    const double tau = tau_s[j], scale = coef[0], beta = coef[1];
-    const int i0 = max(r0, j + 1);                    // my rows below the diagonal
-    double* vj = W + (long long)j * ld - r0;          // vj[i] for global row i
-    const int nc = n - j - 1;                         // trailing columns
-    if (tau != 0.0) {                                 // uniform across the cluster
-      for (int c = j + 1 + tid; c < n; c += nt)
-        wfin[c] = tau * fma(scale, remote_sum(cluster, wpart + b * n + c, C),
-                            *cluster.map_shared_rank(rowj + b * n + c, owner));
-      for (int i = i0 + tid; i < r1; i += nt) vj[i] *= scale;   // local rows only: no hazard with the loads above
-      __syncthreads();
-      for (int t = tid; t < nc * QS; t += nt) {
-        const int c = j + 1 + t / QS, qq = t % QS;
-        double* wc = W + (long long)c * ld - r0;
-        const double w = wfin[c];
-        if (own && qq == 0) wc[j] -= w;
-        axpy_qs(w, vj, wc, i0 + ((qq - i0 % QS + QS) % QS), r1);
+    const double y = ys[j], g = gs[j], h = nb[j];
+    double* wj = W + j * ld - r0;
+    if (j + 1 < n) {
+      // column j+1 first: the pass takes inner products with its new values
+      const double w1 = g * fma(h, rowl[j + 1], dsum[j + 1]);
+      double* w1c = W + (j + 1) * ld - r0;
+      for (int i = max(r0, j + 1) + tid; i < r1; i += nt) w1c[i] = fma(-w1, wj[i], w1c[i]);
+    }
+    for (int c = nt - 1 - tid; c < n; c += nt) {
+      if (c > j + 1) {
+        wfin[c] = g * fma(h, rowl[c], dsum[c]);
+      } else if (c < j) {                             // x_c . x_j
+        tri[j * (j - 1) / 2 + c] = fma(rowl[j] + h, rowl[c], dsum[c]);
       }
-      if (own && tid == 0) vj[j] = beta;
+      if (j % C == rank && c <= j) mc[(j / C) * k + c] = rowl[c];
+    }
+    if (j >= r0 && j < r1 && __double_as_longlong(g) != 0) {   // row j of R
+      for (int c = j + 1 + (nt - 1 - tid); c < n; c += nt) W[c * ld + (j - r0)] = -y * dsum[c];
+      if (tid == 0) wj[j] = -h;
     }
     __syncthreads();
-    if (j + 1 < k) partials(j + 1, 1 - b);
+    if (j + 1 < k) pass(j, j + 1, 1 - b);
   }
-  // R first: Q is formed over W below.
   if (Ro) {
-    for (long long e = tid; e < (long long)rows * n; e += nt) {
-      const int li = int(e % rows), j = int(e / rows), i = r0 + li;
-      if (i < k) Ro[(long long)i * n + j] = (j >= i) ? W[(long long)j * ld + li] : 0.0;
+    for (int e = tid; e < rows * n; e += nt) {
+      const int li = e / n, j = e - li * n, i = r0 + li;
+      if (i < k) Ro[(long long)i * n + j] = (j >= i) ? W[j * ld + li] : 0.0;
     }
+  }
+  for (int j = tid; j < k; j += nt) vs[j] = vs[j] + nb[j];
+  __syncthreads();
+  // X: zero above the diagonal (where R was), alpha - beta on it
+  for (int e = tid; e < rows * k; e += nt) {
+    const int c = e / rows, li = e - c * rows;
+    if (r0 + li <= c) W[c * ld + li] = r0 + li == c ? vs[c] : 0.0;
+  }
+  // M, my columns, one warp each: T^{-1} M = X_1^T from the bottom up
+  for (int cc = tid >> 5; cc < mcols; cc += nt >> 5) {
+    const int c = rank + cc * C;
+    if (c >= k) break;
+    double* x = mc + cc * k;
+    if (lane == 0) x[c] = vs[c];
+    __syncwarp();
+    for (int j = c; j >= 0; --j) {
+      const double* t = tri + j * (j - 1) / 2;
+      const double v = gs[j] * x[j];
+      __syncwarp();
+      for (int i = lane; i < j; i += 32) x[i] = fma(-t[i], v, x[i]);
+      if (lane == 0) x[j] = v;
+      __syncwarp();
+    }
+  }
+  cta_or_cluster_sync();                              // every column of M visible
+  for (int c = tid >> 5; c < k; c += nt >> 5) {
+    double* src = mc + (c / C) * k;
+    if (C > 1) src = cluster.map_shared_rank(src, c % C);
+    for (int i = lane; i <= c; i += 32) tri[c * (c + 1) / 2 + i] = src[i];
   }
   __syncthreads();
-  // Q = H_0 ... H_{k-1} [I_k; 0], formed backwards in place on the same row
-  // split: column j keeps its reflector below the diagonal until step j,
-  // columns c > j already hold Q's columns and are zero in rows <= j.  Rows
-  // above the diagonal (R) are cleared first.
-  for (long long e = tid; e < (long long)rows * k; e += nt) {
-    const int li = int(e % rows), c = int(e / rows);
-    if (r0 + li < c) W[(long long)c * ld + li] = 0.0;
-  }
-  cluster.sync();
-  int nsync = 0;   // double-buffer index: advances only with a cluster barrier
-  for (int j = k - 1; j >= 0; --j) {
-    const double tau = tau_s[j];
-    const bool own = (j >= r0 && j < r1);
-    const int i0 = max(r0, j + 1);
-    double* vj = W + (long long)j * ld - r0;          // vj[i] for global row i
-    const int nc = k - j - 1;                         // columns j+1 .. k-1
-    if (tau != 0.0 && nc > 0) {                       // uniform across the cluster
-      const int b = nsync & 1;
-      ++nsync;
-      for (int t = tid; t < nc * QS; t += nt) {
-        const int c = j + 1 + t / QS, qq = t % QS;
-        const double* qc = W + (long long)c * ld - r0;
-        part4[(long long)c * QS + qq] = dot_qs(vj, qc, i0 + ((qq - i0 % QS + QS) % QS), r1);
-      }
-      __syncthreads();
-      for (int c = j + 1 + tid; c < k; c += nt) {
-        double w = 0.0;
-        for (int qq = 0; qq < QS; ++qq) w += part4[(long long)c * QS + qq];
-        wpart[b * n + c] = w;
-      }
-      cluster.sync();
-      for (int c = j + 1 + tid; c < k; c += nt) wfin[c] = tau * remote_sum(cluster, wpart + b * n + c, C);
-      __syncthreads();
-      for (int t = tid; t < nc * QS; t += nt) {
-        const int c = j + 1 + t / QS, qq = t % QS;
-        double* qc = W + (long long)c * ld - r0;
-        const double w = wfin[c];
-        if (own && qq == 0) qc[j] = -w;
-        axpy_qs(w, vj, qc, i0 + ((qq - i0 % QS + QS) % QS), r1);
-      }
+  // Q = E - X M on my rows, one entry per thread at a time, lanes along rows
+  for (int e = tid; e < rows * k; e += nt) {
+    const int c = e / rows, li = e - c * rows;
+    const double* t = tri + c * (c + 1) / 2;
+    const double* x = W + li;
+    double acc = r0 + li == c ? 1.0 : 0.0;
+    int a = 0;
+    for (; a + 3 <= c; a += 4) {
+      const double x0 = x[a * ld], x1 = x[(a + 1) * ld], x2 = x[(a + 2) * ld], x3 = x[(a + 3) * ld];
+      const double t0 = t[a], t1 = t[a + 1], t2 = t[a + 2], t3 = t[a + 3];
+      acc = fma(-x0, t0, acc);
+      acc = fma(-x1, t1, acc);
+      acc = fma(-x2, t2, acc);
+      acc = fma(-x3, t3, acc);
     }
-    __syncthreads();                                  // every read of the reflector is done
-    for (int i = i0 + tid; i < r1; i += nt) vj[i] *= -tau;
-    if (own && tid == 0) vj[j] = 1.0 - tau;
-    __syncthreads();
+    for (; a <= c; ++a) acc = fma(-x[a * ld], t[a], acc);
+    Qo[(r0 + li) * q.qrs + c * q.qcs] = acc;
   }
-  for (long long e = tid; e < (long long)rows * k; e += nt) {
-    const int li = int(e % rows), c = int(e / rows);
-    Qo[(r0 + li) * q.qrs + c * q.qcs] = W[(long long)c * ld + li];
-  }
-  cluster.sync();   // no CTA leaves while others may still read its shared memory
+  if (C > 1) cluster.sync();   // no CTA leaves while others may still read its shared memory
 }
 
 struct SvdArgs {
@@ -721,75 +823,105 @@ __global__ void __launch_bounds__(SVC_THREADS) k_svd_cluster(const SvdArgs s, do
 }  // namespace
 
 namespace {
-// Largest cluster size (16 non-portable, else 8, 4, 2) with which `kern` can be
-// launched with `smem` bytes of dynamic shared memory per CTA; 1 if clusters
-// are unavailable.  Cached per kernel and size.
+// Clusters of c CTAs of `kern` with `smem` bytes of dynamic shared memory per
+// CTA that run at once; 0 if they cannot be launched.  Cached per kernel,
+// device, threads, size (in 4 KB steps) and c; sets the kernel's attributes.
 template <class K>
-int cluster_size_for(K kern, int threads, size_t smem) {
+int active_clusters(K kern, int threads, size_t smem, int c) {
   static std::mutex mu;
-  static std::vector<std::tuple<const void*, size_t, int>> cache;
-  static std::vector<std::pair<const void*, bool>> attrs;
-  std::lock_guard<std::mutex> g(mu);
+  static std::map<std::tuple<const void*, int, int, size_t, int>, int> cache;
+  static std::map<std::pair<const void*, int>, bool> attrs;
+  int dev = 0;
+  PEPS_CUDA(cudaGetDevice(&dev));
   const void* id = reinterpret_cast<const void*>(kern);
   const size_t key = (smem + 4095) / 4096 * 4096;
-  for (auto& e : cache)
-    if (std::get<0>(e) == id && std::get<1>(e) == key) return std::get<2>(e);
-  bool attrs_ok = false, seen = false;
-  for (auto& a : attrs)
-    if (a.first == id) {
-      attrs_ok = a.second;
-      seen = true;
-    }
-  if (!seen) {
-    attrs_ok = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-               cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess;
+  std::lock_guard<std::mutex> g(mu);
+  const auto k = std::make_tuple(id, dev, threads, key, c);
+  const auto it = cache.find(k);
+  if (it != cache.end()) return it->second;
+  auto at_it = attrs.find({id, dev});
+  if (at_it == attrs.end()) {
+    const bool ok =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024) == cudaSuccess;
     cudaGetLastError();
-    attrs.push_back({id, attrs_ok});
+    at_it = attrs.emplace(std::make_pair(id, dev), ok).first;
   }
-  int best = 1;
-  if (attrs_ok) {
-    for (int c : {16, 8, 4, 2}) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(c, 1, 1);
-      cfg.blockDim = dim3(threads, 1, 1);
-      cfg.dynamicSmemBytes = key;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = c;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      int nclusters = 0;
-      const cudaError_t e = cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg);
-      if (std::getenv("PEPS_VERBOSE"))
-        std::fprintf(stderr, "[peps] qr cluster %d smem %zu: %s, %d active clusters\n", c, key,
-                     cudaGetErrorString(e), nclusters);
-      cudaGetLastError();
-      if (e == cudaSuccess && nclusters > 0) {
-        best = c;
-        break;
-      }
-    }
+  int n = 0;
+  if (at_it->second) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = key;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = c;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+    if (std::getenv("PEPS_VERBOSE"))
+      std::fprintf(stderr, "[peps] cluster %d threads %d smem %zu: %s, %d active clusters\n", c, threads, key,
+                   cudaGetErrorString(e), n);
+    cudaGetLastError();
+    if (e != cudaSuccess) n = 0;
   }
-  cache.push_back(std::make_tuple(id, key, best));
-  return best;
+  cache[k] = n;
+  return n;
 }
 
-int qr_cluster_size(size_t smem) { return cluster_size_for(k_qr_cluster, QRC_THREADS, smem); }
+// Largest cluster size (16 non-portable, else 8, 4, 2) with which `kern` can be
+// launched with `smem` bytes of dynamic shared memory per CTA; 1 if clusters
+// are unavailable.
+template <class K>
+int cluster_size_for(K kern, int threads, size_t smem) {
+  for (int c : {16, 8, 4, 2})
+    if (active_clusters(kern, threads, smem, c) > 0) return c;
+  return 1;
+}
+
 }  // namespace
 
 namespace {
 
-constexpr size_t kQrSmemMax = 200 * 1024;
+// Largest dynamic shared memory of the cluster kernels (227 KB per CTA on sm_103).
+constexpr size_t kQrSmemMax = 224 * 1024;
 
-// Shared memory a cluster QR of an m x n matrix needs per CTA with its rows
-// split over c CTAs (rows of the working matrix and of Q, odd column stride).
+int qr_ld(int m, int c) { return (((m + c - 1) / c) + 7) / 8 * 8 + 4; }   // = 4 mod 8: no bank conflicts
+size_t qr_head_bytes(int m, int n, int c) { return sizeof(double) * size_t(qr_head(n, std::min(m, n), c)); }
+// Shared memory per CTA of an m x n factorisation with its rows split over c
+// CTAs and kept there (the triangle too where that still fits).
 size_t qr_smem(int m, int n, int c) {
-  const int k = std::min(m, n);
-  const size_t base = sizeof(double) * (4 * size_t(n) + 2 + k + size_t(n) * QS + n + 2 + QS);
-  const size_t ld = size_t(((m + c - 1) / c) | 1);
-  return base + sizeof(double) * ld * size_t(n);
+  return qr_head_bytes(m, n, c) + sizeof(double) * size_t(qr_ld(m, c)) * size_t(n);
+}
+// One warp per SM quarter at least; four threads per column while that is no more than 512.
+int qr_threads(int n) { return std::max(128, std::min(QRC_MAXT, (4 * n + 31) / 32 * 32)); }
+
+int qr_lanes_log2(int n) { return n > 16 ? 2 : n > 8 ? 3 : n > 4 ? 4 : 5; }
+
+size_t qr_tri_bytes(int m, int n) { return sizeof(double) * size_t(qr_tri(std::min(m, n))); }
+
+// Estimated clocks of np factorisations on clusters of c CTAs, fitted to
+// measured times of shapes from 16x16 to 2304x64 on 1 to 16 CTAs (within 20%):
+// a column costs its barriers, sums and scalars, its share of the back
+// substitutions, and the FP64 pipe 24 clocks per warp instruction and SM (19
+// at best), two per row and column; the pass leaves a quarter of that idle
+// where a column's warp has an SM quarter to itself, and a triangle in global
+// memory costs a fifth more.  Clusters beyond those that run at once wait:
+// only a few of 16 CTAs do (8192x128 in 8 leaves takes 3.7 ms, in 4 2.9 ms).
+double qr_clocks(int m, int n, int c, int np) {
+  const double k = std::min(m, n), rows = std::ceil(double(m) / c);
+  const double warps = qr_threads(n) / 32;
+  const size_t rows_b = qr_smem(m, n, c), all_b = rows_b + qr_tri_bytes(m, n);
+  const bool tri = all_b <= kQrSmemMax;
+  const int at_once = active_clusters(k_qr_cluster, qr_threads(n), tri ? all_b : rows_b, c);
+  if (at_once == 0) return 1e300;
+  const double step = (c == 1 ? 3800.0 : 5600.0) + 180.0 * std::ceil(std::ceil(k / c) / warps);
+  const double fp = 24.0 * rows * 2.0 * n / 32.0 * (n < 64 ? 1.3 : 1.0);
+  const double waves = std::ceil(double(np) / at_once);
+  const double per_sm = std::ceil(std::min<double>(np, at_once) * c / 148.0);
+  return 10000.0 + waves * k * (step + per_sm * fp) * (tri ? 1.0 : 1.2);
 }
 
 // dst[b][i*qrs + j*qcs] = src[b][i*n + j]
@@ -805,17 +937,105 @@ __global__ void k_copy_strided(const TP src, const TP dst, int m, int n, long lo
   }
 }
 
-// Leaves of a tall-skinny QR: the smallest power of two L >= 2 that divides m
-// and whose leaves (m / L rows, at least 32 per CTA of a 16-CTA cluster)
-// keep their rows in shared memory; 0 if none.
-int tsqr_leaves(int m, int n) {
-  for (int L = 2; L <= 16; L *= 2) {
-    if (m % L) return 0;
-    const int ml = m / L;
-    if (ml < n || ml < 16 * 32) return 0;
-    if (qr_smem(ml, n, 16) <= kQrSmemMax) return L;
+// Largest c (a power of two) up to cmax whose rows fit in shared memory with
+// the least estimated time; 0 if none fits.
+int qr_best_cluster(int m, int n, int np, int cmax, double* clocks) {
+  int best = 0;
+  *clocks = 1e300;
+  for (int c = 1; c <= cmax; c *= 2) {
+    if (qr_smem(m, n, c) > kQrSmemMax) continue;
+    const double t = qr_clocks(m, n, c, np);
+    if (t < *clocks * 1.02) {   // a tie goes to more CTAs
+      *clocks = t;
+      best = c;
+    }
   }
-  return 0;
+  return best;
+}
+
+// How one factorisation runs on k_qr_cluster: cluster size (0: k_qr_house),
+// what is in shared memory, and how much of it.
+struct QrPlan {
+  int C = 0;
+  bool w_smem = false, tri_smem = false;
+  size_t bytes = 0;
+};
+
+// The cluster size with the least estimated time among those whose rows fit in
+// shared memory; rows in global memory, on the largest cluster of 32 rows per
+// CTA or more that still holds the partial sums, where none fits.  Kept per
+// shape (a few integers each): the choice costs several occupancy look-ups.
+QrPlan qr_plan(int m, int n, int np, int qr_cmax) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, int, int, int>, QrPlan> cache;
+  int dev = 0;
+  PEPS_CUDA(cudaGetDevice(&dev));
+  const auto key = std::make_tuple(dev, m, n, np, qr_cmax);
+  {
+    std::lock_guard<std::mutex> g(mu);
+    const auto it = cache.find(key);
+    if (it != cache.end()) return it->second;
+  }
+  const int lim = qr_cmax > 0 ? std::min(qr_cmax, 16) : 16;
+  double clocks;
+  QrPlan p;
+  p.C = qr_best_cluster(m, n, np, lim, &clocks);
+  p.w_smem = p.C > 0;
+  if (!p.w_smem)
+    for (int c = 1; c <= std::min(lim, std::max(1, m / 32)); c *= 2)
+      if (qr_head_bytes(m, n, c) <= kQrSmemMax) p.C = c;
+  auto settle = [&] {
+    const size_t rows = p.w_smem ? qr_smem(m, n, p.C) : qr_head_bytes(m, n, p.C);
+    p.tri_smem = rows + qr_tri_bytes(m, n) <= kQrSmemMax;
+    p.bytes = rows + (p.tri_smem ? qr_tri_bytes(m, n) : 0);
+  };
+  while (p.C > 0) {
+    settle();
+    if (active_clusters(k_qr_cluster, qr_threads(n), p.bytes, p.C) > 0) break;
+    p.C /= 2;   // clusters of this size cannot be launched here
+    p.w_smem = p.C > 0 && qr_smem(m, n, p.C) <= kQrSmemMax;
+    if (p.C > 0 && qr_head_bytes(m, n, p.C) > kQrSmemMax) p.C = 0;
+  }
+  std::lock_guard<std::mutex> g(mu);
+  return cache.emplace(key, p).first->second;
+}
+
+// Leaves of a tall-skinny QR: a power of two L >= 2 that divides m, leaves of
+// at least n rows (and 32 per CTA of a 16-CTA cluster) that fit in shared
+// memory; the one with the least estimated time, 0 if none fits.
+int tsqr_leaves(int m, int n, int np, double* clocks) {
+  int best = 0;
+  *clocks = 1e300;
+  for (int L = 2; L <= 16; L *= 2) {
+    if (m % L || np * L > MAXB) break;
+    const int ml = m / L;
+    if (ml < n || ml < 16 * 32) break;
+    double t1, t2;
+    if (!qr_best_cluster(ml, n, np * L, 16, &t1) || !qr_best_cluster(L * n, n, np, 16, &t2)) continue;
+    const double t = t1 + t2 + 2.0 * double(np) * m * n * n / 148.0 / 3.0 + 20000.0;   // + the Q combine
+    if (t < *clocks) {
+      *clocks = t;
+      best = L;
+    }
+  }
+  return best;
+}
+
+// Leaves of m x n (0: none), kept per shape.
+int tsqr_plan(int m, int n, int np) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, int, int>, int> cache;
+  int dev = 0;
+  PEPS_CUDA(cudaGetDevice(&dev));
+  const auto key = std::make_tuple(dev, m, n, np);
+  std::lock_guard<std::mutex> g(mu);
+  const auto it = cache.find(key);
+  if (it != cache.end()) return it->second;
+  double direct, leaves;
+  qr_best_cluster(m, n, np, 16, &direct);
+  const int L = tsqr_leaves(m, n, np, &leaves);
+  // the estimates are no better than a tenth
+  return cache.emplace(key, L > 1 && leaves < 0.9 * direct ? L : 0).first->second;
 }
 
 }  // namespace
@@ -883,11 +1103,12 @@ void qr_thin(Ctx& cx, int m, int n, const TP& A, long long rs, long long cs, con
   PEPS_REQUIRE(m > 0 && n > 0, "qr of an empty matrix");
   const int np = problems({&A, &Q, &R});
   PEPS_REQUIRE(!A.null() && Q.n == np && (R.null() || R.n == np), "internal: qr operands");
-  // Rows that do not fit in the shared memory of a 16-CTA cluster: tall-skinny
-  // QR over leaves that do (more SMs per factorisation, rows on chip).
-  if (m >= n && cx.qr_cmax <= 0 && qr_smem(m, n, 16) > kQrSmemMax) {
-    const int L = tsqr_leaves(m, n);
-    if (L > 1 && np * L <= MAXB) {
+  // Tall-skinny QR over leaves on more SMs than one cluster has, where the rows
+  // do not fit in the shared memory of one cluster or the leaves are estimated
+  // to be faster.
+  if (m >= 1024 && m >= n && cx.qr_cmax <= 0) {
+    const int L = tsqr_plan(m, n, np);
+    if (L > 1) {
       qr_tsqr(cx, m, n, L, A, rs, cs, Q, qrs, qcs, R, np);
       return;
     }
@@ -899,34 +1120,9 @@ void qr_direct(Ctx& cx, int m, int n, const TP& A, long long rs, long long cs, c
                long long qcs, const TP& R, double counted_flops) {
   const int np = problems({&A, &Q, &R});
   const int k = std::min(m, n);
-  // work of the Householder factorisation with Q formed (for the cluster-size model)
-  const double flops = 4.0 * m * double(n) * k - 4.0 / 3.0 * double(k) * k * k;
-  const size_t base = sizeof(double) * (4 * size_t(n) + 2 + k + size_t(n) * QS + n + 2 + QS);
-  auto ld_of = [&](int c) { return (((m + c - 1) / c) | 1); };   // odd column stride
-  auto full_of = [&](int c) { return qr_smem(m, n, c); };
-  // Cluster size: rows per CTA >= 32; among the sizes whose rows fit in shared
-  // memory, the one with the least estimated time for all problems: waves of
-  // clusters over the SMs x (FP64 work per CTA + three cluster barriers per column).
-  int cmax = std::max(1, std::min(cx.qr_cmax > 0 ? cx.qr_cmax : 16, m / 32));
-  while (cmax > 1 && (cmax & (cmax - 1))) --cmax;
-  int C = cmax;
-  if (cmax > 1) {
-    double best = 1e300;
-    for (int c = 2; c <= cmax; c *= 2) {
-      if (full_of(c) > kQrSmemMax && c < cmax) continue;
-      const double waves = std::ceil(double(np) * c / 144.0);
-      const double t = waves * (flops / (c * 8.0e9) + 3.0 * k * 1.5e-6);
-      if (t < best) {
-        best = t;
-        C = c;
-      }
-    }
-    C = std::min(C, qr_cluster_size(full_of(C) <= kQrSmemMax ? full_of(C) : base));
-    while (C > 1 && (C & (C - 1))) --C;
-  }
+  const QrPlan pl = qr_plan(m, n, np, cx.qr_cmax);
+  const int C = pl.C;
   if (std::getenv("PEPS_VERBOSE")) std::fprintf(stderr, "[peps] qr %dx%d x%d: cluster %d\n", m, n, np, C);
-  const int ld = ld_of(std::max(C, 1));
-  const bool in_smem = C > 1 && full_of(C) <= kQrSmemMax;
   QrArgs a;
   std::memset(static_cast<void*>(&a), 0, sizeof(a));
   a.m = m;
@@ -938,26 +1134,29 @@ void qr_direct(Ctx& cx, int m, int n, const TP& A, long long rs, long long cs, c
   a.qrs = qrs;
   a.qcs = qcs;
   a.R = R.all(np);
-  if (C <= 1) {
+  const int ld = qr_ld(m, std::max(C, 1));
+  const long long tri = qr_tri(k);
+  if (C == 0) {
     a.wst = (long long)m * n;
     a.qst = (long long)m * k;
-  } else {   // the global-memory fallback uses [C][n][ld] blocks per problem (Q formed in place)
-    a.wst = (long long)C * ld * n;
-    a.qst = 0;
+    a.tst = k;
+  } else if (!pl.w_smem || !pl.tri_smem) {
+    a.wst = C * ((pl.tri_smem ? 0 : tri) + (pl.w_smem ? 0 : (long long)ld * n));
   }
-  a.tst = k;
-  double* w = cx.scratch(size_t(np) * (a.wst + a.qst + a.tst) + 64);
-  a.W = w;
-  a.Qw = w + size_t(np) * a.wst;
-  a.tau = a.Qw + size_t(np) * a.qst;
+  if (a.wst) {
+    double* w = cx.scratch(size_t(np) * (a.wst + a.qst + a.tst) + 64);
+    a.W = w;
+    a.Qw = w + size_t(np) * a.wst;
+    a.tau = a.Qw + size_t(np) * a.qst;
+  }
   Launch L(K_QR, cx.st, counted_flops, 0);
-  if (C <= 1) {
+  if (C == 0) {
     k_qr_house<<<np, QR_THREADS, 0, cx.st>>>(a);
   } else {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C * np, 1, 1);
-    cfg.blockDim = dim3(QRC_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = in_smem ? full_of(C) : base;
+    cfg.blockDim = dim3(qr_threads(n), 1, 1);
+    cfg.dynamicSmemBytes = pl.bytes;
     cfg.stream = cx.st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -966,7 +1165,7 @@ void qr_direct(Ctx& cx, int m, int n, const TP& A, long long rs, long long cs, c
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    PEPS_CUDA(cudaLaunchKernelEx(&cfg, k_qr_cluster, a, in_smem ? 1 : 0, ld));
+    PEPS_CUDA(cudaLaunchKernelEx(&cfg, k_qr_cluster, a, pl.w_smem ? 1 : 0, pl.tri_smem ? 1 : 0, ld, qr_lanes_log2(n)));
   }
   PEPS_CHECK_LAUNCH();
 }

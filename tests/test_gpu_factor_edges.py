@@ -1,0 +1,29 @@
+"""The FP64 factorisations at the edges of their size rules, through the norm
+sweep against the FP64 oracle (tolerance as in test_gpu_parity: 1e-10 absolute
+on ln N)."""
+import pytest
+
+from oracle import peps_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def peps():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1311_6696_gb300 import peps as P
+    return P
+
+
+# Shapes of the QR's boundary tensors, rows x columns: one CTA (12x3), ragged
+# rows over a cluster (175x7), more columns than four threads each cover and a
+# triangle in global memory (1620x180), tall-skinny candidates (1188x33).
+@pytest.mark.parametrize("Ly,Lx,D,chi,mode", [(4, 6, 2, 3, "var"), (4, 4, 5, 7, "var"), (4, 5, 3, 20, "svd"),
+                                              (4, 4, 6, 33, "var")])
+def test_norm_at_factor_edges(peps, Ly, Lx, D, chi, mode):
+    from paper_1311_6696_gb300 import synth
+    A = synth.peps_gauss(Ly, Lx, 2, D, seed=40 + D)
+    got, want = peps.norm(A, chi, mode=mode, seed=2), O.norm(A, chi=chi, mode=mode, seed=2)
+    assert abs(got[0] - want[0]) < 1e-10 and got[1] == want[1]
