@@ -1,5 +1,5 @@
-"""The FP64 factorisations at the edges of their size rules, through the norm
-sweep against the FP64 oracle (tolerance as in test_gpu_parity: 1e-10 absolute
+"""The FP64 factorisations and contractions at the edges of their size rules,
+through the norm sweep against the FP64 oracle (tolerance as in test_gpu_parity: 1e-10 absolute
 on ln N)."""
 import pytest
 
@@ -19,9 +19,12 @@ def peps():
 
 # Shapes of the QR's boundary tensors, rows x columns: one CTA (12x3), ragged
 # rows over a cluster (175x7), more columns than four threads each cover and a
-# triangle in global memory (1620x180), tall-skinny candidates (1188x33).
+# triangle in global memory (1620x180), tall-skinny candidates (1188x33).  The
+# last three are for the contractions: one-element groups and K below a tile
+# (D = 1, chi = 1), ragged tiles with K split over a cluster (D = 7, chi = 5).
 @pytest.mark.parametrize("Ly,Lx,D,chi,mode", [(4, 6, 2, 3, "var"), (4, 4, 5, 7, "var"), (4, 5, 3, 20, "svd"),
-                                              (4, 4, 6, 33, "var")])
+                                              (4, 4, 6, 33, "var"), (3, 5, 1, 4, "var"),
+                                              (4, 3, 3, 1, "var"), (4, 4, 7, 5, "var")])
 def test_norm_at_factor_edges(peps, Ly, Lx, D, chi, mode):
     from paper_1311_6696_gb300 import synth
     A = synth.peps_gauss(Ly, Lx, 2, D, seed=40 + D)
