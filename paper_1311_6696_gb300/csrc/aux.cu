@@ -1,5 +1,7 @@
 // Auxiliary kernels: lattice repacking, OBC validation, norms and rescaling,
 // counter-based var initialisation, local observables and CU_0.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -7,6 +9,8 @@
 
 #include "aux.cuh"
 #include "linalg.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace peps {
 namespace {
@@ -579,6 +583,261 @@ __global__ void __launch_bounds__(256) k_cu0(const Cu0Lattice* lats, int* flag) 
   }
 }
 
+
+// ----------------------------------------------------------------------------
+// CU_0 in two kernels per row.
+//
+// The row's ALS is a serial chain over its sites, and on one CTA (k_cu0) every
+// local update pays four O(d D^5) contractions at one SM's FP64 rate, 60 us at
+// D = 6.  Everything in them but the two environments and the matrix being
+// fitted is fixed during the fit, so k_cu0_build first contracts, for all
+// sites of the row in parallel, the site pair with the matrix above it into
+//   H[no][lm][rq] = sum over orders of (l,m), (n,o), (r,q) of
+//                   sum_{s,u,v} S[u,v] A[s,u,l,n,r] A[s,v,m,o,q],
+// pairs taken once (l <= m ...): environments and closures are symmetric, so
+// T = D (D + 1) / 2 entries stand for D^2 and H has T^3 of D^6.  With
+// w = 1 on the diagonal and 2 off it, an update is b[no] = L H[no] R / w[no],
+// and the next environment sum_no b[no] (L H[no])[rq] / w[rq] takes the same
+// product L H[no] (b's norm drops out when that is normalised): one T^3
+// contraction per site and half-sweep instead of eight of d D^5.
+// k_cu0_als then runs the fit on a cluster of C CTAs per side, each with its
+// share of the no's, one exchange per update: the CTA's b's and its part of
+// the environment.  A chain of ~6,000 clocks per update (exchange, three
+// reductions over a warp, one reciprocal root) bounds it.
+// ----------------------------------------------------------------------------
+constexpr int CU0_MAXD = 8;
+constexpr int CU0_MAXT = CU0_MAXD * (CU0_MAXD + 1) / 2;
+constexpr int CU0_THREADS = 256;
+
+__host__ __device__ inline int tri_count(int n) { return n * (n + 1) / 2; }
+
+// pi <= pj of packed pair p = pj (pj + 1) / 2 + pi, the same for every dimension.
+__device__ __forceinline__ void pair_tables(int* pi, int* pj) {
+  if (threadIdx.x < CU0_MAXT) {
+    const int p = threadIdx.x;
+    int j = 0;
+    while ((j + 1) * (j + 2) / 2 <= p) ++j;
+    pj[p] = j;
+    pi[p] = p - j * (j + 1) / 2;
+  }
+}
+
+// Grid = (sites x parts, lattices): H of the sites of row r, the no's of one part.
+__global__ void __launch_bounds__(CU0_THREADS) k_cu0_build(const Cu0Lattice* lats, int r, int parts) {
+  extern __shared__ double bsm[];
+  __shared__ int pi[CU0_MAXT], pj[CU0_MAXT];
+  const Cu0Lattice L = lats[blockIdx.y];
+  const int x = blockIdx.x / parts, part = blockIdx.x % parts;
+  if (r + 1 >= L.Ly || x >= L.Lx) return;
+  const int tid = threadIdx.x, nt = blockDim.x, d = L.d, DM2 = L.Dmax * L.Dmax;
+  const int* dm = L.dims + 4 * (r * L.Lx + x);
+  const int du = dm[0], dl = dm[1], dn = dm[2], dr = dm[3], P3 = dl * dn * dr, K = d * du;
+  const double* S = r == 0 ? L.top + (long long)x * DM2 : L.out + ((long long)r * L.Lx + x) * DM2;
+  const double* Ag = L.A + L.off[r * L.Lx + x];
+  double* A = bsm;              // [s][u][l][n][r]
+  double* B = bsm + K * P3;     // [s][v][l][n][r] = sum_u S[u,v] A
+  pair_tables(pi, pj);
+  for (int e = tid; e < K * P3; e += nt) A[e] = Ag[e];
+  __syncthreads();
+  for (int e = tid; e < K * P3; e += nt) {
+    const int sv = e / P3, o = e - sv * P3, s = sv / du, v = sv - s * du;
+    const double* a = A + s * du * P3 + o;
+    double acc = 0.0;
+    for (int u = 0; u < du; ++u) acc = fma(S[u * du + v], a[u * P3], acc);
+    B[e] = acc;
+  }
+  __syncthreads();
+  const int Tl = tri_count(dl), Tn = tri_count(dn), Tr = tri_count(dr);
+  const int T0 = tri_count(L.Dmax);
+  double* H = L.work + (long long)x * 2 * T0 * T0 * T0;   // [no][lm][rq], then [no][rq][lm]
+  double* Ht = H + (long long)T0 * T0 * T0;
+  const int per = (Tn + parts - 1) / parts, no1 = min(Tn, (part + 1) * per);
+  for (int e = part * per * Tl * Tr + tid; e < no1 * Tl * Tr; e += nt) {
+    const int no = e / (Tl * Tr), lr = e - no * Tl * Tr, lm = lr / Tr, rq = lr - lm * Tr;
+    const int n = pi[no], o = pj[no], l = pi[lm], m = pj[lm], rr = pi[rq], q = pj[rq];
+    const int bl = (l * dn + n) * dr, bm = (m * dn + n) * dr, al = (l * dn + o) * dr, am = (m * dn + o) * dr;
+    double acc = 0.0;
+    for (int k = 0; k < K; ++k) {
+      const double* b = B + k * P3;
+      const double* a = A + k * P3;
+      acc = fma(b[bl + rr], a[am + q], acc);
+      acc = fma(b[bm + rr], a[al + q], acc);
+      acc = fma(b[bl + q], a[am + rr], acc);
+      acc = fma(b[bm + q], a[al + rr], acc);
+    }
+    // four orders of (l,m) and (r,q); equal ones were counted twice
+    const double f = (l == m ? 0.5 : 1.0) * (rr == q ? 0.5 : 1.0) * (n == o ? 1.0 : 2.0);
+    H[(no * Tl + lm) * Tr + rq] = f * acc;
+    Ht[(no * Tr + rq) * Tl + lm] = f * acc;
+  }
+}
+
+// The fit of the matrices below row r; one cluster of C CTAs per lattice.
+__global__ void __launch_bounds__(CU0_THREADS) k_cu0_als(const Cu0Lattice* lats, int r, int* flag) {
+  extern __shared__ double asm_[];
+  __shared__ int pi[CU0_MAXT], pj[CU0_MAXT];
+  __shared__ double pub[2][2 * CU0_MAXT];                  // my b's, then my part of the next environment
+  __shared__ double vec[CU0_THREADS / 32 + CU0_MAXT][CU0_MAXT];
+  __shared__ double bs[CU0_MAXT], braw[CU0_MAXT], eraw[CU0_MAXT];
+  __shared__ int s_conv;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = int(cluster.num_blocks()), rank = int(cluster.block_rank());
+  const Cu0Lattice Lt = lats[blockIdx.x / C];
+  if (r + 1 >= Lt.Ly) return;                              // the whole cluster
+  const int Lx = Lt.Lx, DM2 = Lt.Dmax * Lt.Dmax, T0 = tri_count(Lt.Dmax);
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  double* Le = asm_;                    // [Lx][T0] left environments, packed
+  double* Re = Le + Lx * T0;
+  double* N = Re + Lx * T0;             // [Lx][T0] the matrices being fitted
+  auto dims = [&](int x) { return Lt.dims + 4 * (r * Lx + x); };
+  pair_tables(pi, pj);
+  __syncthreads();
+  for (int x = 0; x < Lx; ++x) {        // identity start, unit Frobenius norm
+    const int dn = dims(x)[2];
+    const double v = 1.0 / sqrt(double(dn));
+    for (int e = tid; e < tri_count(dn); e += nt) N[x * T0 + e] = pi[e] == pj[e] ? v : 0.0;
+  }
+  {
+    const int dr = dims(Lx - 1)[3], dl = dims(0)[1];
+    for (int e = tid; e < tri_count(dr); e += nt)
+      Re[(Lx - 1) * T0 + e] = Lt.right[(long long)r * DM2 + pi[e] * dr + pj[e]];
+    for (int e = tid; e < tri_count(dl); e += nt) Le[e] = Lt.left[(long long)r * DM2 + pi[e] * dl + pj[e]];
+  }
+  __syncthreads();
+  int phase = 0;
+  double change = 0.0;                  // warp 0: largest squared movement of this half-sweep
+  // One site.  dir 0: left environment in, right one out; 1: the reverse.
+  // update: N[x] is refitted first; env: the next environment is formed.
+  auto site = [&](int x, int dir, bool update, bool env) {
+    const int* dm = dims(x);
+    const int Tl = tri_count(dm[1]), Tn = tri_count(dm[2]), Tr = tri_count(dm[3]);
+    const int Ti = dir == 0 ? Tl : Tr, To = dir == 0 ? Tr : Tl;
+    const double* vin = (dir == 0 ? Le : Re) + x * T0;
+    const double* vo = (dir == 0 ? Re : Le) + x * T0;
+    const double* H = Lt.work + (long long)x * 2 * T0 * T0 * T0 + (dir == 0 ? 0 : (long long)T0 * T0 * T0);
+    const int per = (Tn + C - 1) / C, n0 = min(Tn, rank * per), mine = min(Tn, n0 + per) - n0;
+    const int P = mine > 0 ? max(1, nw / mine) : 1, chunk = (Ti + P - 1) / P;   // warps per no
+    for (int t = warp; t < mine * P; t += nw) {
+      const int k = t / P, p = t - k * P, i1 = min(Ti, (p + 1) * chunk);
+      const double* h = H + (long long)(n0 + k) * Ti * To;
+      for (int o = lane; o < To; o += 32) {
+        double acc = 0.0;
+#pragma unroll 6
+        for (int i = p * chunk; i < i1; ++i) acc = fma(vin[i], h[i * To + o], acc);
+        vec[t][o] = acc;
+      }
+    }
+    __syncthreads();
+    for (int k = warp; k < mine; k += nw) {
+      double s = 0.0;
+      for (int o = lane; o < To; o += 32) {
+        double v = vec[k * P][o];
+        for (int p = 1; p < P; ++p) v += vec[k * P + p][o];
+        vec[k * P][o] = v;
+        s = fma(v, vo[o], s);
+      }
+      if (update) {
+        s = warp_sum(s);
+        if (pi[n0 + k] != pj[n0 + k]) s *= 0.5;
+      } else {
+        s = N[x * T0 + n0 + k];
+      }
+      if (lane == 0) bs[k] = s;
+    }
+    __syncthreads();
+    double* mypub = pub[phase];
+    if (tid < mine) mypub[tid] = bs[tid];
+    if (env) {
+      for (int o = nt - 1 - tid; o < To; o += nt) {
+        double v = 0.0;
+        for (int k = 0; k < mine; ++k) v = fma(bs[k], vec[k * P][o], v);
+        mypub[CU0_MAXT + o] = v;
+      }
+    }
+    if (C > 1)
+      cluster.sync();
+    else
+      __syncthreads();
+    if (update)
+      for (int e = tid; e < Tn; e += nt)
+        braw[e] = C > 1 ? *cluster.map_shared_rank(mypub + e % per, e / per) : mypub[e];
+    if (env)
+      for (int o = nt - 1 - tid; o < To; o += nt) {
+        double v[8], sum = 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = q < C ? *cluster.map_shared_rank(mypub + CU0_MAXT + o, q) : 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (q < C) sum += v[q];
+        eraw[o] = pi[o] == pj[o] ? sum : 0.5 * sum;
+      }
+    phase ^= 1;
+    __syncthreads();
+    // unit Frobenius norm (off-diagonal entries count twice); zero stays zero
+    auto unit = [&](const double* v, int n) {
+      double s = 0.0;
+      for (int e = lane; e < n; e += 32) s = fma(pi[e] == pj[e] ? v[e] : 2.0 * v[e], v[e], s);
+      s = warp_sum(s);
+      return s > 0.0 ? rsqrt(s) : 0.0;
+    };
+    if (warp == 0 && update) {
+      const double inv = unit(braw, Tn);
+      double c = 0.0;
+      for (int e = lane; e < Tn; e += 32) {
+        const double v = braw[e] * inv, df = v - N[x * T0 + e];
+        N[x * T0 + e] = v;
+        c = fma(pi[e] == pj[e] ? df : 2.0 * df, df, c);
+      }
+      change = fmax(change, warp_sum(c));
+    } else if (warp == 1 && env) {
+      const double inv = unit(eraw, To);
+      double* out = dir == 0 ? Le + (x + 1) * T0 : Re + (x - 1) * T0;
+      for (int e = lane; e < To; e += 32) out[e] = eraw[e] * inv;
+    }
+    __syncthreads();
+  };
+  for (int x = Lx - 1; x >= 1; --x) site(x, 1, false, true);
+  bool conv = false;
+  for (int h = 0; h < Lt.max_half && !conv; ++h) {
+    change = 0.0;
+    for (int step = 0; step < Lx; ++step) {
+      const int x = (h % 2 == 0) ? step : Lx - 1 - step;
+      site(x, h % 2, true, step + 1 < Lx);
+    }
+    if (tid == 0) s_conv = change < Lt.tol * Lt.tol;       // the same in every CTA: same sums, same order
+    __syncthreads();
+    conv = s_conv != 0;
+  }
+  if (!conv && tid == 0 && rank == 0) atomicOr(flag, FLAG_CU0_NOCONV);
+  for (int x = rank; x < Lx; x += C) {
+    const int dn = dims(x)[2];
+    double* out = Lt.out + ((long long)(r + 1) * Lx + x) * DM2;
+    for (int e = tid; e < dn * dn; e += nt) {
+      const int i = min(e / dn, e % dn), j = max(e / dn, e % dn);
+      out[e] = N[x * T0 + j * (j + 1) / 2 + i];
+    }
+  }
+  if (C > 1) cluster.sync();   // no CTA leaves while others may still read its shared memory
+}
+
+// Row 0 of every lattice: the closures above it.
+__global__ void k_cu0_top(const Cu0Lattice* lats) {
+  const Cu0Lattice L = lats[blockIdx.x];
+  const int DM2 = L.Dmax * L.Dmax;
+  for (int x = 0; x < L.Lx; ++x) {
+    const int du = L.dims[4 * x];
+    for (int e = threadIdx.x; e < du * du; e += blockDim.x) L.out[(long long)x * DM2 + e] = L.top[(long long)x * DM2 + e];
+  }
+}
+
+// Shared memory of the two kernels for a lattice; the fast path needs both to fit.
+size_t cu0_build_smem(int d, int D) { return sizeof(double) * 2 * size_t(d) * D * D * D * D; }
+size_t cu0_als_smem(int Lx, int D) { return sizeof(double) * 3 * size_t(Lx) * tri_count(D); }
+constexpr size_t kCu0Smem = 180 * 1024;
+bool cu0_fast(int Lx, int d, int D) {
+  return D <= CU0_MAXD && cu0_build_smem(d, D) <= kCu0Smem && cu0_als_smem(Lx, D) <= kCu0Smem;
+}
+
 }  // namespace
 
 void orient_lattice(Ctx& cx, const void* src, int src_f32, int /*Ly*/, int Lx, int d, int D,
@@ -735,14 +994,57 @@ void copy(Ctx& cx, const TP& dst, const TP& src, long long n) {
 }
 
 size_t cu0_work_size(int Lx, int d, int Dmax) {
-  const size_t D2 = size_t(Dmax) * Dmax;
+  const size_t D2 = size_t(Dmax) * Dmax, T = size_t(tri_count(Dmax));
+  if (cu0_fast(Lx, d, Dmax)) return 2 * size_t(Lx) * T * T * T;
   return 2 * size_t(d) * D2 * D2 + 2 * size_t(Lx) * D2 + D2;
 }
 
 void cu0_launch(Ctx& cx, const Cu0Lattice* lats, int nlat) {
   auto* dev = static_cast<const Cu0Lattice*>(stage(cx, lats, sizeof(Cu0Lattice) * nlat));
+  int Ly = 1, Lx = 1, D = 1, d = 1;
+  bool fast = true;
+  for (int i = 0; i < nlat; ++i) {
+    Ly = std::max(Ly, lats[i].Ly);
+    Lx = std::max(Lx, lats[i].Lx);
+    D = std::max(D, lats[i].Dmax);
+    d = std::max(d, lats[i].d);
+    fast = fast && cu0_fast(lats[i].Lx, lats[i].d, lats[i].Dmax);
+  }
   Launch L(K_CU0, cx.st);
-  k_cu0<<<nlat, 256, 0, cx.st>>>(dev, cx.flag);
+  if (!fast) {   // D > 8, or rows too long for shared memory: one CTA per side
+    k_cu0<<<nlat, 256, 0, cx.st>>>(dev, cx.flag);
+    PEPS_CHECK_LAUNCH();
+    return;
+  }
+  static std::once_flag once;
+  std::call_once(once, [] {
+    PEPS_CUDA(cudaFuncSetAttribute(k_cu0_build, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCu0Smem)));
+    PEPS_CUDA(cudaFuncSetAttribute(k_cu0_als, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCu0Smem)));
+  });
+  const int T = tri_count(D);
+  // Parts per site: about two CTAs per SM, no part without a no.
+  const int parts = std::max(1, std::min(T, 2 * 152 / std::max(1, Lx * nlat)));
+  // Up to T = 10 (D = 4) a row's products take one SM about as long as the
+  // exchange between several.
+  const int C = T <= 10 ? 1 : 8;
+  k_cu0_top<<<nlat, 128, 0, cx.st>>>(dev);
+  for (int r = 0; r + 1 < Ly; ++r) {
+    k_cu0_build<<<dim3(Lx * parts, nlat), CU0_THREADS, cu0_build_smem(d, D), cx.st>>>(dev, r, parts);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C * nlat, 1, 1);
+    cfg.blockDim = dim3(CU0_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = cu0_als_smem(Lx, D);
+    cfg.stream = cx.st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    PEPS_CUDA(cudaLaunchKernelEx(&cfg, k_cu0_als, dev, r, cx.flag));
+    L.more(2);
+  }
   PEPS_CHECK_LAUNCH();
 }
 
