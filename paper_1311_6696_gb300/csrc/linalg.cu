@@ -1,9 +1,8 @@
 // FP64 Householder QR and one-sided Jacobi SVD, batched over independent
 // problems of one shape.
 //
-// Small matrices take one CTA each (working copy in global memory, L2
-// resident; one warp per column reduction).  Larger ones are split by rows
-// over a thread-block cluster of 2-16 CTAs that exchange partial sums through
+// A matrix is split by rows over a thread-block cluster of 1-16 CTAs, kept in
+// shared memory where it fits, and the CTAs exchange partial sums through
 // distributed shared memory: the QR with one cluster barrier per Householder
 // column, the SVD with one per round of the round-robin Jacobi schedule.
 #include <cooperative_groups.h>
@@ -26,7 +25,6 @@ namespace peps {
 namespace {
 
 constexpr int QR_THREADS = 512;
-constexpr int SVD_THREADS = 512;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -486,301 +484,258 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
 }
 
 struct SvdArgs {
-  int p, q;          // working matrix G is p x q (p >= q), column-major
-  int m, n;          // original A is m x n row-major
-  int trans;         // 1: G = A^T (m < n)
+  int p, q;          // G is p x q (p >= q), G(i, j) = A[i*rs + j*cs]
   TP A;              // per problem
-  double* work;      // per problem (+ problem * wst): G (p x q), V (q x q), nrm (q), order (q ints)
-  long long wst;
+  long long rs, cs;
+  int trans;         // 1: the SVD of G^T is wanted, else that of G
+  double* work;      // rows of G and V where shared memory does not hold them
+  long long wst;     // doubles of work per problem
   int kk;
-  TP US;             // m x kk row-major
-  TP Vt;             // kk x n row-major
+  TP US;             // (trans ? q : p) x kk row-major
+  TP Vt;             // kk x (trans ? p : q) row-major
   int* flag;
   int max_sweeps;    // sweep cap (PEPS_ECONVERGE when reached)
 };
 
-// Grid = problems, one CTA each.
-__global__ void __launch_bounds__(SVD_THREADS) k_svd_jacobi(const SvdArgs s) {
-  __shared__ int s_rot;
-  const int p = s.p, q = s.q;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-  const int pb = blockIdx.x;
-  const double* A = s.A.d(pb);
-  double* const US = s.US.d(pb);
-  double* const Vto = s.Vt.d(pb);
-  double* G = s.work + pb * s.wst;
-  double* V = G + (long long)p * q;
-  double* const nrm = V + (long long)q * q;
-  int* const order = reinterpret_cast<int*>(nrm + q);
-  for (long long e = tid; e < (long long)p * q; e += nt) {
-    int i = int(e % p), j = int(e / p);   // G(i,j)
-    G[e] = s.trans ? A[(long long)j * s.n + i] : A[(long long)i * s.n + j];
-  }
-  for (long long e = tid; e < (long long)q * q; e += nt) V[e] = ((e % q) == (e / q)) ? 1.0 : 0.0;
-  __syncthreads();
-  const int qq = q + (q & 1);   // even number of slots for the round-robin pairing
-  // a pair is orthogonal once |gamma| <= tol sqrt(alpha beta); rounding alone
-  // leaves |gamma| / sqrt(alpha beta) of order p * eps after a rotation, so the
-  // threshold scales with the row count (as in LAPACK's one-sided Jacobi)
-  const double tol = fmax(1e-15, 4.0 * double(p) * 2.220446049250313e-16);
-  int sweep = 0;
-  for (; sweep < s.max_sweeps; ++sweep) {
-    if (tid == 0) s_rot = 0;
-    __syncthreads();
-    for (int round = 0; round < qq - 1; ++round) {
-      for (int pr = warp; pr < qq / 2; pr += nw) {
-        // round-robin (circle) schedule: slot 0 fixed, others rotate
-        int a = (pr == 0) ? 0 : 1 + (pr - 1 + round) % (qq - 1);
-        int b = 1 + (qq - 2 - pr + round) % (qq - 1);
-        if (a >= q || b >= q) continue;
-        if (a > b) { int t = a; a = b; b = t; }
-        double al = 0.0, be = 0.0, ga = 0.0;
-        const double* ga_ = G + (long long)a * p;
-        const double* gb_ = G + (long long)b * p;
-        for (int i = lane; i < p; i += 32) {
-          double x = ga_[i], y = gb_[i];
-          al += x * x;
-          be += y * y;
-          ga += x * y;
-        }
-        al = warp_sum(al);
-        be = warp_sum(be);
-        ga = warp_sum(ga);
-        if (ga != 0.0 && fabs(ga) > tol * sqrt(al * be)) {
-          const double zeta = (be - al) / (2.0 * ga);
-          const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-          const double c = 1.0 / sqrt(1.0 + t * t), sn = c * t;
-          double* gA = G + (long long)a * p;
-          double* gB = G + (long long)b * p;
-          for (int i = lane; i < p; i += 32) {
-            double x = gA[i], y = gB[i];
-            gA[i] = c * x - sn * y;
-            gB[i] = sn * x + c * y;
-          }
-          double* vA = V + (long long)a * q;
-          double* vB = V + (long long)b * q;
-          for (int i = lane; i < q; i += 32) {
-            double x = vA[i], y = vB[i];
-            vA[i] = c * x - sn * y;
-            vB[i] = sn * x + c * y;
-          }
-          if (lane == 0) s_rot = 1;
-        }
-      }
-      __syncthreads();
-    }
-    const int rot = s_rot;
-    __syncthreads();
-    if (!rot) break;
-  }
-  if (sweep >= s.max_sweeps && tid == 0) atomicOr(s.flag, FLAG_SVD_NOCONV);
-  // column norms and a stable descending order
-  for (int j = warp; j < q; j += nw) {
-    double v = 0.0;
-    for (int i = lane; i < p; i += 32) {
-      double x = G[(long long)j * p + i];
-      v += x * x;
-    }
-    v = warp_sum(v);
-    if (lane == 0) nrm[j] = sqrt(v);
-  }
-  __syncthreads();
-  for (int j = tid; j < q; j += nt) {
-    const double vj = nrm[j];
-    int r = 0;
-    for (int i = 0; i < q; ++i) {
-      const double vi = nrm[i];
-      r += (vi > vj) || (vi == vj && i < j);
-    }
-    order[r] = j;
-  }
-  __syncthreads();
-  // A V = G  (A = G V^T when trans = 0;  A^T = G V^T  =>  A = V G^T when trans = 1)
-  const int kk = s.kk;
-  if (!s.trans) {
-    // US[i][r] = G(i, order[r]);  Vt[r][j] = V(j, order[r])
-    for (long long e = tid; e < (long long)s.m * kk; e += nt) {
-      int i = int(e / kk), r = int(e % kk);
-      US[e] = (r < q) ? G[(long long)order[r] * p + i] : 0.0;
-    }
-    for (long long e = tid; e < (long long)kk * s.n; e += nt) {
-      int r = int(e / s.n), j = int(e % s.n);
-      Vto[e] = (r < q) ? V[(long long)order[r] * q + j] : 0.0;
-    }
-  } else {
-    // US[i][r] = V(i, order[r]) * nrm;  Vt[r][j] = G(j, order[r]) / nrm
-    for (long long e = tid; e < (long long)s.m * kk; e += nt) {
-      int i = int(e / kk), r = int(e % kk);
-      US[e] = (r < q) ? V[(long long)order[r] * q + i] * nrm[order[r]] : 0.0;
-    }
-    for (long long e = tid; e < (long long)kk * s.n; e += nt) {
-      int r = int(e / s.n), j = int(e % s.n);
-      double nr = (r < q) ? nrm[order[r]] : 0.0;
-      Vto[e] = (r < q && nr > 0.0) ? G[(long long)order[r] * p + j] / nr : 0.0;
-    }
+// ---------------------------------------------------------------------------
+// One-sided Jacobi (Hestenes) on a thread-block cluster of C = 1-16 CTAs: the
+// rows of the working matrix G (p x q) and of V (q x q) are split over the
+// CTAs and kept in shared memory where they fit.  A round of the round-robin
+// schedule rotates q / 2 disjoint column pairs.
+//
+// What bounds it: the FP64 pipe (64 clocks per warp instruction and SM
+// quarter) and, for the matrices of a boundary fit, the chain of one round --
+// inner products, cluster barrier, sums, rotation scalars, rotation.  So
+//   * one inner product per pair and round: squared column norms are exact at
+//     the start of a sweep and follow the rotations inside it
+//     (alpha' = alpha - t gamma, beta' = beta + t gamma); a sweep without
+//     rotations, the one that ends the iteration, has tested exact norms;
+//   * t comes from FP32: a rotation only has to be orthogonal to working
+//     precision -- c = 1 / sqrt(1 + t^2) is, in FP64, for the t that is used --
+//     and one that leaves 1e-7 of the inner product is finished by the next
+//     sweep like any other remainder;
+//   * scaled rotations (fast Givens): columns are kept as G = G' diag(d), and
+//     a rotation is one FMA per element, g_a' -= t d_b / d_a g_b',
+//     g_b' += t d_a / d_b g_a' (old values), d *= c; d goes back into the
+//     columns every 64 rounds;
+//   * partial sums stay in their CTA and are read after the barrier.
+// Same threshold, ordering and output rules as LAPACK's one-sided Jacobi: a
+// pair is orthogonal once |gamma| <= tol sqrt(alpha beta) with
+// tol = 4 p eps (rounding alone leaves p eps).
+// Measured (us; before: plain rotations and three inner products per pair and
+// round, rows in global memory): random 16x16 579 -> 252, 32 of 64x64 6178 ->
+// 3141, 180x180 42059 -> 13997, without the preconditioning of svd_trunc; with it
+// 32 of 64x64 3128, 180x180 12338, graded 180x180 27617 -> 8014.  A round of
+// 180x180 is now 13,000 clocks: the rotations take half of it, the scalars a
+// third.
+// ---------------------------------------------------------------------------
+constexpr int SVC_MAXT = 512;
+constexpr int SVC_RESCALE = 64;
+
+__host__ __device__ inline long long svd_head(int q) {
+  const long long npair = (q + 1) / 2;
+  return 4 * npair + 3LL * q + 2 * npair + q + (q + 1) / 2 + 2;
+}
+__host__ __device__ inline int svd_ld(int rows) { return rows | 1; }   // odd: no bank conflicts across columns
+
+// Slots (a, b) of pair pr in a round of the circle schedule over qq slots: slot 0 fixed, the others rotate.
+__device__ __forceinline__ void jacobi_pair(int pr, int round, int qq, int& a, int& b) {
+  const int w = qq - 1;
+  int u = pr - 1 + round, v = qq - 2 - pr + round;
+  u -= u >= w ? w : 0;
+  v -= v >= w ? w : 0;
+  a = pr == 0 ? 0 : 1 + u;
+  b = 1 + v;
+  if (a > b) {
+    const int t = a;
+    a = b;
+    b = t;
   }
 }
 
-// ---------------------------------------------------------------------------
-// One-sided Jacobi on a thread-block cluster: the rows of the working matrix G
-// (p x q) and of V (q x q) are split over the cluster's CTAs.  A round of the
-// round-robin schedule is one cluster barrier: every CTA publishes its partial
-// (alpha, beta, gamma) of every pair, then sums all CTAs' partials in the same
-// order -- so every CTA forms the same rotations -- and rotates its own rows.
-// Same rotations, threshold, ordering and output as the one-CTA kernel.
-// ---------------------------------------------------------------------------
-constexpr int SVC_THREADS = 256;
+// 1 / sqrt(x) for x in [1, 2]: one cubic step from the FP32 value.
+__device__ __forceinline__ double rsqrt_1to2(double x) {
+  const double y = double(rsqrtf(float(x)));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
 
-__global__ void __launch_bounds__(SVC_THREADS) k_svd_cluster(const SvdArgs s, double* work, long long wst) {
+// x * 2^k by the exponent bits; 0 below the normal range.
+__device__ __forceinline__ double scale2(double x, int k) {
+  const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+  if (ex == 0 || ex + k <= 0) return 0.0;
+  return __hiloint2double(hi + k * (1 << 20), __double2loint(x));
+}
+
+__global__ void __launch_bounds__(SVC_MAXT) k_svd_cluster(const SvdArgs s, int head_smem, int rows_smem, int lanes_log2) {
   extern __shared__ double ssm[];
   cg::cluster_group cluster = cg::this_cluster();
   const int C = int(cluster.num_blocks()), rank = int(cluster.block_rank());
   const int pb = blockIdx.x / C;
-  const int p = s.p, q = s.q, tid = threadIdx.x, nt = blockDim.x;
+  const int p = s.p, q = s.q, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   const int qq = q + (q & 1), npair = qq / 2;
   const int cp = (p + C - 1) / C, cv = (q + C - 1) / C;
-  const int g0 = min(p, rank * cp), g1 = min(p, g0 + cp), gr = g1 - g0;   // my rows of G
-  const int v0 = min(q, rank * cv), v1 = min(q, v0 + cv), vr = v1 - v0;   // my rows of V
-  double* part = ssm;                         // [2][3][npair] my partial sums (cluster-visible)
-  double* cs = part + 6 * npair;              // [2][2][npair] rotation (c, s) of this round
-  double* nrm = cs + 4 * npair;               // [q]
+  const int g0 = min(p, rank * cp), gr = min(p, g0 + cp) - g0;            // my rows of G
+  const int v0 = min(q, rank * cv), vr = min(q, v0 + cv) - v0;            // my rows of V
+  const int ld = svd_ld(cp + cv);             // a column: my rows of G, then (at cp) my rows of V
+  double* const work = s.work + pb * s.wst + rank * (s.wst / C);
+  double* part = head_smem ? ssm : work;      // [2][2 npair] my partial sums (read by every CTA)
+  double* al = part + 4 * npair;              // [q] squared norms
+  double* ds = al + q;                        // [q] column scales
+  double* es = ds + q;                        // [q] their reciprocals
+  double* ta = es + q;                        // [npair] this round's rotations: t d_b / d_a
+  double* tb = ta + npair;                    // [npair] t d_a / d_b
+  double* nrm = tb + npair;                   // [q]
   int* order = reinterpret_cast<int*>(nrm + q);   // [q]
   __shared__ int s_rot;
-  double* G = work + pb * wst + (long long)rank * cp * q;                   // [q][cp] column-major block
-  double* V = work + pb * wst + (long long)C * cp * q + (long long)rank * cv * q;   // [q][cv]
+  double* G = rows_smem ? ssm + svd_head(q) : work + (head_smem ? 0 : svd_head(q));
   const double* A = s.A.d(pb);
+  const bool rows_first = s.rs < s.cs;
   for (long long e = tid; e < (long long)gr * q; e += nt) {
-    const int li = int(e % gr), j = int(e / gr), i = g0 + li;
-    G[(long long)j * cp + li] = s.trans ? A[(long long)j * s.n + i] : A[(long long)i * s.n + j];
+    const int j = int(rows_first ? e / gr : e % q), li = int(rows_first ? e % gr : e / q);
+    G[(long long)j * ld + li] = A[(g0 + li) * s.rs + j * s.cs];
   }
-  for (long long e = tid; e < (long long)vr * q; e += nt) {
-    const int li = int(e % vr), j = int(e / vr);
-    V[(long long)j * cv + li] = (v0 + li == j) ? 1.0 : 0.0;
+  for (int j = warp; j < q; j += nw)
+    for (int li = lane; li < vr; li += 32) G[(long long)j * ld + cp + li] = (v0 + li == j) ? 1.0 : 0.0;
+  for (int j = tid; j < q; j += nt) {
+    ds[j] = 1.0;
+    es[j] = 1.0;
   }
-  // a pair is orthogonal once |gamma| <= tol sqrt(alpha beta); rounding alone
-  // leaves |gamma| / sqrt(alpha beta) of order p * eps after a rotation, so the
-  // threshold scales with the row count (as in LAPACK's one-sided Jacobi)
-  const double tol = fmax(1e-15, 4.0 * double(p) * 2.220446049250313e-16);
-  int sweep = 0, t = 0;
-  for (; sweep < s.max_sweeps; ++sweep) {
-    int rotated = 0;
-    for (int round = 0; round < qq - 1; ++round, ++t) {
-      const int b = t & 1;
-      __syncthreads();
-      for (int pr = tid; pr < npair; pr += nt) {
-        int a = (pr == 0) ? 0 : 1 + (pr - 1 + round) % (qq - 1);
-        int c = 1 + (qq - 2 - pr + round) % (qq - 1);
-        if (a > c) {
-          const int tmp = a;
-          a = c;
-          c = tmp;
-        }
-        double al = 0.0, be = 0.0, ga = 0.0;
-        if (a < q && c < q) {
-          const double* xa = G + (long long)a * cp;
-          const double* xc = G + (long long)c * cp;
-          for (int i = 0; i < gr; ++i) {
-            const double x = xa[i], y = xc[i];
-            al = fma(x, x, al);
-            be = fma(y, y, be);
-            ga = fma(x, y, ga);
-          }
-        }
-        part[(b * 3 + 0) * npair + pr] = al;
-        part[(b * 3 + 1) * npair + pr] = be;
-        part[(b * 3 + 2) * npair + pr] = ga;
-      }
+  auto cta_or_cluster_sync = [&]() {
+    if (C > 1)
       cluster.sync();
+    else
+      __syncthreads();
+  };
+  auto sum_parts = [&](double* slot) { return C > 1 ? remote_sum(cluster, slot, C) : *slot; };
+  // the scales into the columns (after a barrier; followed by one)
+  auto rescale = [&]() {
+    for (int j = warp; j < q; j += nw) {
+      const double d = ds[j];
+      double* x = G + (long long)j * ld;
+      for (int li = lane; li < cp + vr; li += 32)
+        if (li < gr || li >= cp) x[li] *= d;
+    }
+    __syncthreads();
+    for (int j = tid; j < q; j += nt) {
+      ds[j] = 1.0;
+      es[j] = 1.0;
+    }
+  };
+  int buf = 0;   // double-buffer index of part: advances with every exchange
+  // exact squared norms of the columns into al
+  auto norms = [&]() {
+    for (int j = warp; j < q; j += nw) {
+      const double* x = G + (long long)j * ld;
+      double v = 0.0;
+      for (int li = lane; li < gr; li += 32) v = fma(x[li], x[li], v);
+      v = warp_sum(v);
+      if (lane == 0) part[buf * 2 * npair + j] = v;
+    }
+    cta_or_cluster_sync();
+    for (int j = tid; j < q; j += nt) al[j] = sum_parts(part + buf * 2 * npair + j);
+    buf ^= 1;
+    __syncthreads();
+  };
+  const double tol = fmax(1e-15, 4.0 * double(p) * 2.220446049250313e-16);
+  const int sh = lanes_log2, L = 1 << sh;   // threads per inner product
+  const int W = cp + vr > 16 ? 32 : (cp + vr > 8 ? 16 : 8);   // lanes per rotated pair
+  __syncthreads();
+  int sweep = 0;
+  for (; sweep < s.max_sweeps; ++sweep) {
+    rescale();
+    if (tid == 0) s_rot = 0;
+    __syncthreads();
+    norms();
+    int rotated = 0;
+    for (int round = 0; round < qq - 1; ++round) {
+      if (round % SVC_RESCALE == SVC_RESCALE - 1) {
+        rescale();
+        __syncthreads();
+      }
+      for (int t0 = tid - lane; t0 < npair << sh; t0 += nt) {
+        const int pr = (t0 + lane) >> sh, l = lane & (L - 1);
+        int a, b;
+        jacobi_pair(pr, round, qq, a, b);
+        double ga = 0.0;
+        if (pr < npair && b < q) {
+          const double* xa = G + (long long)a * ld;
+          const double* xb = G + (long long)b * ld;
+#pragma unroll 4
+          for (int li = l; li < gr; li += L) ga = fma(xa[li], xb[li], ga);
+        }
+        for (int o = L >> 1; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+        if (pr < npair && l == 0) part[buf * 2 * npair + pr] = ga;
+      }
+      cta_or_cluster_sync();
       for (int pr = tid; pr < npair; pr += nt) {
-        int a = (pr == 0) ? 0 : 1 + (pr - 1 + round) % (qq - 1);
-        int c = 1 + (qq - 2 - pr + round) % (qq - 1);
-        double cc = 1.0, sn = 0.0;
-        if (a < q && c < q) {
-          if (a > c) {
-            const int tmp = a;
-            a = c;
-            c = tmp;
-          }
-          // all 3C remote loads in flight before any add (one round trip), summed in rank order
-          double va[16], vb[16], vg[16];
-#pragma unroll
-          for (int r = 0; r < 16; ++r) {
-            va[r] = r < C ? *cluster.map_shared_rank(part + (b * 3 + 0) * npair + pr, r) : 0.0;
-            vb[r] = r < C ? *cluster.map_shared_rank(part + (b * 3 + 1) * npair + pr, r) : 0.0;
-            vg[r] = r < C ? *cluster.map_shared_rank(part + (b * 3 + 2) * npair + pr, r) : 0.0;
-          }
-          double al = 0.0, be = 0.0, ga = 0.0;
-#pragma unroll
-          for (int r = 0; r < 16; ++r) {
-            al += va[r];
-            be += vb[r];
-            ga += vg[r];
-          }
-          if (ga != 0.0 && fabs(ga) > tol * sqrt(al * be)) {
-            const double zeta = (be - al) / (2.0 * ga);
-            const double tt = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-            cc = 1.0 / sqrt(1.0 + tt * tt);
-            sn = cc * tt;
+        int a, b;
+        jacobi_pair(pr, round, qq, a, b);
+        double x = 0.0, y = 0.0;
+        if (b < q) {
+          const double da = ds[a], db = ds[b], A2 = al[a], B2 = al[b];
+          const double ga = sum_parts(part + buf * 2 * npair + pr) * da * db;
+          // gamma^2 > tol^2 alpha beta, tested on the sign of the difference
+          const double over = fma(-(tol * A2), tol * B2, ga * ga);
+          if (__double2hiint(over) > 0 || (__double2hiint(over) == 0 && __double2loint(over) != 0)) {
+            const double dl = B2 - A2;
+            const int k = 1023 - ((max(__double2hiint(A2), __double2hiint(B2)) >> 20) & 0x7ff);
+            const float df = float(scale2(dl, k)), gf = 2.f * float(scale2(ga, k));
+            double t;
+            if (fabsf(gf) > 1e-18f) {
+              const float h = fabsf(df) + sqrtf(fmaf(df, df, gf * gf));
+              t = double(df >= 0.f ? gf / h : -gf / h);
+              if (df == 0.f) t = 1.0;
+            } else {
+              t = ga / dl;   // far apart: the angle itself, beyond FP32's range
+            }
+            const double w = fma(t, t, 1.0), c = rsqrt_1to2(w), ic = w * c;
+            x = t * (db * es[a]);
+            y = t * (da * es[b]);
+            al[a] = fma(-t, ga, A2);
+            al[b] = fma(t, ga, B2);
+            ds[a] = da * c;
+            ds[b] = db * c;
+            es[a] *= ic;
+            es[b] *= ic;
             rotated = 1;
           }
         }
-        cs[(b * 2 + 0) * npair + pr] = cc;
-        cs[(b * 2 + 1) * npair + pr] = sn;
+        ta[pr] = x;
+        tb[pr] = y;
+      }
+      buf ^= 1;
+      __syncthreads();
+      // rotate my rows of G and V
+      const int sub = lane / W, per = 32 / W;
+      for (int pr = warp * per + sub; pr < npair; pr += nw * per) {
+        const double x = ta[pr], y = tb[pr];
+        if (__double_as_longlong(x) << 1 == 0 && __double_as_longlong(y) << 1 == 0) continue;
+        int a, b;
+        jacobi_pair(pr, round, qq, a, b);
+        double* xa = G + (long long)a * ld;
+        double* xb = G + (long long)b * ld;
+        for (int li = lane & (W - 1); li < cp + vr; li += W) {
+          if (li >= gr && li < cp) continue;
+          const double u = xa[li], v = xb[li];
+          xa[li] = fma(-x, v, u);
+          xb[li] = fma(y, u, v);
+        }
       }
       __syncthreads();
-      // rotate my rows of G and V: consecutive threads take consecutive rows of one pair
-      for (long long e = tid; e < (long long)npair * (gr + vr); e += nt) {
-        const int row = int(e % (gr + vr)), pr = int(e / (gr + vr));
-        const double cc = cs[(b * 2 + 0) * npair + pr], sn = cs[(b * 2 + 1) * npair + pr];
-        if (sn == 0.0) continue;
-        int a = (pr == 0) ? 0 : 1 + (pr - 1 + round) % (qq - 1);
-        int c = 1 + (qq - 2 - pr + round) % (qq - 1);
-        if (a > c) {
-          const int tmp = a;
-          a = c;
-          c = tmp;
-        }
-        double* X;
-        int ld, li;
-        if (row < gr) {
-          X = G;
-          ld = cp;
-          li = row;
-        } else {
-          X = V;
-          ld = cv;
-          li = row - gr;
-        }
-        const double x = X[(long long)a * ld + li], y = X[(long long)c * ld + li];
-        X[(long long)a * ld + li] = cc * x - sn * y;
-        X[(long long)c * ld + li] = sn * x + cc * y;
-      }
     }
-    if (tid == 0) s_rot = 0;
-    __syncthreads();
     if (rotated) s_rot = 1;   // benign race: every writer stores 1
     __syncthreads();
-    if (!s_rot) break;        // identical in every CTA (same sums, same decisions)
+    const int rot = s_rot;
+    __syncthreads();
+    if (!rot) break;          // identical in every CTA (same sums, same decisions)
   }
   if (sweep >= s.max_sweeps && tid == 0 && rank == 0) atomicOr(s.flag, FLAG_SVD_NOCONV);
   // column norms of G over all rows, then a stable descending order
-  cluster.sync();
-  const int b = t & 1;
-  for (int j = tid; j < q; j += nt) {
-    const double* x = G + (long long)j * cp;
-    double v = 0.0;
-    for (int i = 0; i < gr; ++i) v = fma(x[i], x[i], v);
-    nrm[j] = v;
-  }
+  rescale();
   __syncthreads();
-  // publish squared norms through the part buffer (size 3*npair >= q)
-  for (int j = tid; j < q; j += nt) part[b * 3 * npair + j] = nrm[j];
-  cluster.sync();
-  for (int j = tid; j < q; j += nt) {
-    double v = 0.0;
-    v = remote_sum(cluster, part + b * 3 * npair + j, C);
-    nrm[j] = sqrt(v);
-  }
+  norms();
+  for (int j = tid; j < q; j += nt) nrm[j] = sqrt(al[j]);
   __syncthreads();
   for (int j = tid; j < q; j += nt) {
     const double vj = nrm[j];
@@ -795,29 +750,31 @@ __global__ void __launch_bounds__(SVC_THREADS) k_svd_cluster(const SvdArgs s, do
   const int kk = s.kk;
   double* const US = s.US.d(pb);
   double* const Vt = s.Vt.d(pb);
+  const int n = s.trans ? p : q;
+  // G0 V = G: G0 = G V^T, G0^T = V G^T
   if (!s.trans) {
     // US[i][r] = G(i, order[r]) for my G rows; Vt[r][j] = V(j, order[r]) for my V rows
-    for (long long e = tid; e < (long long)gr * kk; e += nt) {
-      const int li = int(e / kk), r = int(e % kk);
-      US[(long long)(g0 + li) * kk + r] = (r < q) ? G[(long long)order[r] * cp + li] : 0.0;
+    for (int e = tid; e < gr * kk; e += nt) {
+      const int li = e / kk, r = e % kk;
+      US[(long long)(g0 + li) * kk + r] = (r < q) ? G[(long long)order[r] * ld + li] : 0.0;
     }
-    for (long long e = tid; e < (long long)vr * kk; e += nt) {
-      const int li = int(e / kk), r = int(e % kk);
-      if (r < kk) Vt[(long long)r * s.n + (v0 + li)] = (r < q) ? V[(long long)order[r] * cv + li] : 0.0;
+    for (int e = tid; e < vr * kk; e += nt) {
+      const int r = e / vr, li = e % vr;
+      Vt[(long long)r * n + (v0 + li)] = (r < q) ? G[(long long)order[r] * ld + cp + li] : 0.0;
     }
   } else {
     // US[i][r] = V(i, order[r]) * nrm for my V rows; Vt[r][j] = G(j, order[r]) / nrm for my G rows
-    for (long long e = tid; e < (long long)vr * kk; e += nt) {
-      const int li = int(e / kk), r = int(e % kk);
-      US[(long long)(v0 + li) * kk + r] = (r < q) ? V[(long long)order[r] * cv + li] * nrm[order[r]] : 0.0;
+    for (int e = tid; e < vr * kk; e += nt) {
+      const int li = e / kk, r = e % kk;
+      US[(long long)(v0 + li) * kk + r] = (r < q) ? G[(long long)order[r] * ld + cp + li] * nrm[order[r]] : 0.0;
     }
-    for (long long e = tid; e < (long long)gr * kk; e += nt) {
-      const int li = int(e / kk), r = int(e % kk);
+    for (int e = tid; e < gr * kk; e += nt) {
+      const int r = e / gr, li = e % gr;
       const double nr = (r < q) ? nrm[order[r]] : 0.0;
-      Vt[(long long)r * s.n + (g0 + li)] = (r < q && nr > 0.0) ? G[(long long)order[r] * cp + li] / nr : 0.0;
+      Vt[(long long)r * n + (g0 + li)] = (r < q && nr > 0.0) ? G[(long long)order[r] * ld + li] / nr : 0.0;
     }
   }
-  cluster.sync();   // no CTA leaves while others may still read its shared memory
+  if (C > 1) cluster.sync();   // no CTA leaves while others may still read its shared memory
 }
 
 }  // namespace
@@ -869,16 +826,6 @@ int active_clusters(K kern, int threads, size_t smem, int c) {
   }
   cache[k] = n;
   return n;
-}
-
-// Largest cluster size (16 non-portable, else 8, 4, 2) with which `kern` can be
-// launched with `smem` bytes of dynamic shared memory per CTA; 1 if clusters
-// are unavailable.
-template <class K>
-int cluster_size_for(K kern, int threads, size_t smem) {
-  for (int c : {16, 8, 4, 2})
-    if (active_clusters(kern, threads, smem, c) > 0) return c;
-  return 1;
 }
 
 }  // namespace
@@ -1170,58 +1117,110 @@ void qr_direct(Ctx& cx, int m, int n, const TP& A, long long rs, long long cs, c
   PEPS_CHECK_LAUNCH();
 }
 
-void svd_trunc(Ctx& cx, int m, int n, const TP& A, int kk, const TP& US, const TP& Vt) {
-  PEPS_REQUIRE(m > 0 && n > 0 && kk > 0, "svd of an empty matrix");
-  const int np = problems({&A, &US, &Vt});
-  PEPS_REQUIRE(!A.null() && US.n == np && Vt.n == np, "internal: svd operands");
+// Jacobi SVD of G (or G^T), see SvdArgs.
+void svd_jacobi(Ctx& cx, int p, int q, const TP& A, long long rs, long long cs, int trans, int kk, const TP& US,
+                const TP& Vt, int np) {
   SvdArgs s;
   std::memset(static_cast<void*>(&s), 0, sizeof(s));
-  s.trans = (m < n) ? 1 : 0;
-  s.p = s.trans ? n : m;
-  s.q = s.trans ? m : n;
-  s.m = m;
-  s.n = n;
+  s.p = p;
+  s.q = q;
   s.A = A.all(np);
+  s.rs = rs;
+  s.cs = cs;
+  s.trans = trans;
   s.kk = kk;
   s.US = US.all(np);
   s.Vt = Vt.all(np);
   s.flag = cx.flag;
   s.max_sweeps = std::max(1, cx.svd_cap);
-  s.wst = ((long long)s.p * s.q + (long long)s.q * s.q + 2LL * s.q + 31) / 32 * 32;
-  s.work = cx.scratch(size_t(np) * s.wst);
-  const double flops = 8.0 * 4.0 * double(s.p) * s.q * s.q;
-  // Matrices of 4096+ entries: rows split over a thread-block cluster (16 rows per CTA or more).
+  // Cluster size: the least estimated time.  A round costs its barriers, sums
+  // and scalars, and the FP64 pipe's share of 3 p + 2 q FMAs per pair; clusters
+  // beyond those that run at once wait, several CTAs on an SM share its pipe.
+  const int npair = (s.q + 1) / 2, nt = npair > 64 ? 512 : npair > 32 ? 256 : 128;
+  const size_t head = sizeof(double) * size_t(svd_head(s.q));
+  auto rows_of = [&](int c) { return size_t(svd_ld((s.p + c - 1) / c + (s.q + c - 1) / c)) * s.q; };
   int C = 1;
-  if (double(s.p) * s.q >= 4096.0) {
-    C = std::max(1, std::min(16, s.p / 16));
-    while (C > 1 && (C & (C - 1))) --C;
+  bool head_smem = false, rows_smem = false;
+  double best = 1e300;
+  for (int c = 1; c <= 16 && head <= kQrSmemMax; c *= 2) {
+    const bool fits = head + sizeof(double) * rows_of(c) <= kQrSmemMax;
+    const size_t smem = head + (fits ? sizeof(double) * rows_of(c) : 0);
+    if (c > 1 && s.p / c < 2) break;
+    const int at_once = active_clusters(k_svd_cluster, nt, smem, c);
+    if (at_once == 0) continue;
+    const double per_sm = std::max(1.0, double(std::min(np, at_once)) * c / 148.0);
+    const double round = (c == 1 ? 2400.0 : 3600.0 + 70.0 * c) +
+                         per_sm * (fits ? 1.0 : 2.0) * npair * (3.0 * s.p + 2.0 * s.q) / (1.4 * c);
+    const double t = std::ceil(double(np) / at_once) * round;
+    if (t < best) {
+      best = t;
+      C = c;
+      head_smem = true;
+      rows_smem = fits;
+    }
   }
-  const int npair = (s.q + (s.q & 1)) / 2;
-  const size_t smem = sizeof(double) * (10 * size_t(npair) + s.q + (s.q + 1) / 2 + 8);
-  if (C > 1) C = std::min(C, cluster_size_for(k_svd_cluster, SVC_THREADS, smem));
-  while (C > 1 && (C & (C - 1))) --C;
-  Launch L(K_SVD, cx.st, flops * np, 0);
-  if (C <= 1) {
-    k_svd_jacobi<<<np, SVD_THREADS, 0, cx.st>>>(s);
-  } else {
-    const int cp = (s.p + C - 1) / C, cv = (s.q + C - 1) / C;
-    const long long cwst = (long long)C * cp * s.q + (long long)C * cv * s.q;
-    double* cwork = cx.scratch(size_t(np) * cwst + 64);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C * np, 1, 1);
-    cfg.blockDim = dim3(SVC_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = cx.st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    PEPS_CUDA(cudaLaunchKernelEx(&cfg, k_svd_cluster, s, cwork, cwst));
+  // (a matrix too wide for even its sums in shared memory runs on one CTA from global memory)
+  if (!head_smem || !rows_smem) {
+    s.wst = C * ((head_smem ? 0 : svd_head(s.q)) + (rows_smem ? 0 : (long long)rows_of(C)));
+    s.work = cx.scratch(size_t(np) * s.wst + 64);
   }
+  const int rows = (s.p + C - 1) / C;
+  int lanes = 0;   // threads per inner product: up to 8, while each has four rows and a thread to itself
+  while (lanes < 3 && (npair << (lanes + 1)) <= nt && (rows >> (lanes + 1)) >= 4) ++lanes;
+  Launch L(K_SVD, cx.st, 0, 0);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(C * np, 1, 1);
+  cfg.blockDim = dim3(nt, 1, 1);
+  cfg.dynamicSmemBytes = (head_smem ? head : 0) + (rows_smem ? sizeof(double) * rows_of(C) : 0);
+  cfg.stream = cx.st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  PEPS_CUDA(cudaLaunchKernelEx(&cfg, k_svd_cluster, s, head_smem ? 1 : 0, rows_smem ? 1 : 0, lanes));
   PEPS_CHECK_LAUNCH();
+}
+
+// From this width on the iteration runs on a matrix preconditioned by two QR
+// factorisations (Drmac & Veselic, without pivoting): G = Q1 R1, R1^T = Q2 R2,
+// so G = Q1 R2^T Q2^T, and R2^T is close to diagonal.  The centre matrices of
+// a boundary, whose singular values fall by 10 to 20 orders, take 14 to 40
+// sweeps as they are and 7 or 8 so (180x180: 28 and 40 sweeps -> 8); random ones
+// 10 and 8.  Below, the four extra launches cost what the sweeps do.
+constexpr int SVD_PRECOND = 12;
+
+void svd_trunc(Ctx& cx, int m, int n, const TP& A, int kk, const TP& US, const TP& Vt) {
+  PEPS_REQUIRE(m > 0 && n > 0 && kk > 0, "svd of an empty matrix");
+  const int np = problems({&A, &US, &Vt});
+  PEPS_REQUIRE(!A.null() && US.n == np && Vt.n == np, "internal: svd operands");
+  const int trans = m < n ? 1 : 0, p = trans ? n : m, q = trans ? m : n;
+  const long long rs = trans ? 1 : n, cs = trans ? n : 1;
+  {
+    Launch count(K_SVD, cx.st, 8.0 * 4.0 * double(p) * q * q * np, 0);   // the flops, once; launches count themselves
+    count.more(-1);
+  }
+  if (q < SVD_PRECOND || kk > q) {
+    svd_jacobi(cx, p, q, A, rs, cs, trans, kk, US, Vt, np);
+    return;
+  }
+  const size_t qq = size_t(q) * q, pq = size_t(p) * q, qk = size_t(q) * kk;
+  auto up = [](size_t x) { return (x + 31) / 32 * 32; };
+  Arena tmp(cx.st, sizeof(double) * np * (up(pq) + 3 * up(qq) + 2 * up(qk)));
+  auto blk = [&](size_t per) { return strided(tmp.dalloc(up(per) * np), np, per); };
+  const TP Q1 = blk(pq), R1 = blk(qq), Q2 = blk(qq), R2 = blk(qq), u = blk(qk), v = blk(qk);
+  qr_thin(cx, p, q, A, rs, cs, Q1, q, 1, R1);
+  qr_thin(cx, q, q, R1, 1, q, Q2, q, 1, R2);
+  svd_jacobi(cx, q, q, R2, 1, q, trans, kk, u, v, np);
+  // G = Q1 (u v) Q2^T, G^T = Q2 (u v) Q1^T
+  cx.f64_class = K_SVD;
+  cx.f64_flops = false;
+  ein(cx, "iq,qk->ik", trans ? Q2 : Q1, {trans ? q : p, q}, u, {q, kk}, US);
+  ein(cx, "kq,iq->ki", v, {kk, q}, trans ? Q1 : Q2, {trans ? p : q, q}, Vt);
+  cx.f64_class = -1;
+  cx.f64_flops = true;
 }
 
 }  // namespace peps

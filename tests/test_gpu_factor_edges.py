@@ -20,11 +20,14 @@ def peps():
 # Shapes of the QR's boundary tensors, rows x columns: one CTA (12x3), ragged
 # rows over a cluster (175x7), more columns than four threads each cover and a
 # triangle in global memory (1620x180), tall-skinny candidates (1188x33).  The
-# last three are for the contractions: one-element groups and K below a tile
+# next three are for the contractions: one-element groups and K below a tile
 # (D = 1, chi = 1), ragged tiles with K split over a cluster (D = 7, chi = 5).
+# The last are for the SVD: fewer columns than its preconditioning takes (9),
+# wider than high and higher than wide (27x81, 81x27), odd widths (49).
 @pytest.mark.parametrize("Ly,Lx,D,chi,mode", [(4, 6, 2, 3, "var"), (4, 4, 5, 7, "var"), (4, 5, 3, 20, "svd"),
                                               (4, 4, 6, 33, "var"), (3, 5, 1, 4, "var"),
-                                              (4, 3, 3, 1, "var"), (4, 4, 7, 5, "var")])
+                                              (4, 3, 3, 1, "var"), (4, 4, 7, 5, "var"),
+                                              (4, 4, 3, 1, "svd"), (3, 5, 3, 9, "svd"), (3, 4, 7, 7, "svd")])
 def test_norm_at_factor_edges(peps, Ly, Lx, D, chi, mode):
     from paper_1311_6696_gb300 import synth
     A = synth.peps_gauss(Ly, Lx, 2, D, seed=40 + D)
