@@ -13,6 +13,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <cuda.h>
 #include <functional>
 #include <map>
 #include <memory>
@@ -127,6 +128,57 @@ int fault_from_env() {
 }
 int cap_cu0_half_sweeps() { return g_cap_cu0.load(); }
 int cap_jacobi_sweeps() { return g_cap_jacobi.load(); }
+
+namespace {
+constexpr cuuint64_t kPoolKeep = 4ull << 30;
+
+// The library's memory pool of a device; nullptr where the device has none.
+cudaMemPool_t device_pool(int dev) {
+  static std::mutex mu;
+  static std::map<int, cudaMemPool_t> pools;
+  std::lock_guard<std::mutex> g(mu);
+  auto it = pools.find(dev);
+  if (it != pools.end()) return it->second;
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.handleTypes = cudaMemHandleTypeNone;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  cudaMemPool_t pool = nullptr;
+  cuuint64_t keep = kPoolKeep;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) pool = nullptr;
+  if (pool) cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  cudaGetLastError();
+  pools[dev] = pool;
+  return pool;
+}
+}  // namespace
+
+cudaError_t pool_alloc(void** p, size_t n, cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  int dev = 0;
+  cudaMemPool_t pool = nullptr;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+      cudaGetDevice(&dev) == cudaSuccess)
+    pool = device_pool(dev);
+  else
+    cudaGetLastError();
+  if (!pool) return cudaMallocAsync(p, n, st);
+  cudaError_t e = cudaMallocFromPoolAsync(p, n, pool, st);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(p, n, pool, st);
+  }
+  return e;
+}
+
+void pool_trim() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return;
+  if (cudaMemPool_t pool = device_pool(dev)) cudaMemPoolTrimTo(pool, 0);
+  cudaGetLastError();
+}
 
 int peps_set_error(int code, const std::string& msg) { return fail(code, msg); }
 
@@ -400,7 +452,12 @@ void build_orientations(Ctx& cx, const peps_lattice* in, Arena& keep, Oriented& 
 std::unique_ptr<peps_env> new_env(const peps_lattice* lat, int kind, cudaStream_t st) {
   auto env = std::make_unique<peps_env>();
   PEPS_CUDA(cudaGetDevice(&env->device));
-  env->arena = std::make_unique<Arena>(st, size_t(64) << 20, /*async=*/false);
+  // chunks of about what the handle will hold (four oriented copies of the
+  // lattice and as much in boundaries), 2 to 64 MB: mapping and unmapping 64 MB
+  // would be most of a small call's host time
+  const size_t lattice = size_t(lat->Ly) * lat->Lx * lat->d * lat->D * lat->D * lat->D * lat->D * sizeof(double);
+  const size_t chunk = std::min<size_t>(size_t(64) << 20, std::max<size_t>(size_t(2) << 20, 8 * lattice));
+  env->arena = std::make_unique<Arena>(st, chunk, /*async=*/false);
   env->kind = kind;
   EnvData& e = env->data;
   e.Ly = lat->Ly;

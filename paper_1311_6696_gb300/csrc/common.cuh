@@ -88,12 +88,24 @@ int cap_cu0_half_sweeps();
 int cap_jacobi_sweeps();
 extern std::atomic<int> g_fault_alloc;      // > 0 while a PEPS_FAULT=alloc call runs
 
+// Stream-ordered device allocation (freed with cudaFreeAsync) from the
+// library's own memory pool of the current device.  The pool keeps up to 4 GB
+// of freed memory mapped between calls -- the device's default pool unmaps
+// everything at each synchronisation, and mapping the workspaces again took
+// 2 to 3 ms of a small call -- and gives the rest back at the next
+// synchronisation, all of it when an allocation of the library fails.  While
+// the stream is being captured the allocation becomes a memory node of the
+// graph.  Safe from several threads and streams, as cudaMallocAsync is.
+cudaError_t pool_alloc(void** p, size_t n, cudaStream_t st);
+// Returns the pool's kept memory to the device.
+void pool_trim();
+
 // ---------------------------------------------------------------------------
-// Stream-ordered bump arena (cudaMallocAsync chunks, freed together).
+// Stream-ordered bump arena (pool_alloc chunks, freed together).
 // ---------------------------------------------------------------------------
 class Arena {
  public:
-  // async: chunks come from cudaMallocAsync on `st` and are freed stream-ordered;
+  // async: chunks come from pool_alloc on `st` and are freed stream-ordered;
   // otherwise cudaMalloc / cudaFree (for memory that outlives the caller's stream).
   explicit Arena(cudaStream_t st, size_t chunk = size_t(64) << 20, bool async = true)
       : st_(st), chunk_(chunk), async_(async) {}
@@ -110,7 +122,12 @@ class Arena {
     if (bytes > left_) {
       size_t n = bytes > chunk_ ? bytes : chunk_;
       void* p = nullptr;
-      cudaError_t e = async_ ? cudaMallocAsync(&p, n, st_) : cudaMalloc(&p, n);
+      cudaError_t e = async_ ? pool_alloc(&p, n, st_) : cudaMalloc(&p, n);
+      if (e != cudaSuccess && !async_) {   // what the pool keeps may be what is missing
+        cudaGetLastError();
+        pool_trim();
+        e = cudaMalloc(&p, n);
+      }
       if (e != cudaSuccess) {
         cudaGetLastError();
         throw Error(PEPS_ENOMEM, std::string("device allocation of ") + std::to_string(n) +

@@ -41,7 +41,7 @@ struct Ctx {
       if (scr) cudaFreeAsync(scr, st);
       size_t m = n + n / 4 + 1024;
       void* p = nullptr;
-      cudaError_t e = cudaMallocAsync(&p, m * sizeof(double), st);
+      cudaError_t e = pool_alloc(&p, m * sizeof(double), st);
       if (e != cudaSuccess) {
         cudaGetLastError();
         scr = nullptr;
