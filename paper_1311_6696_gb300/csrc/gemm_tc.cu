@@ -40,9 +40,17 @@ constexpr int TC_STAGES = 4;
 constexpr int TC_ROWB = 128;          // bytes per tile row = one 128-byte swizzle row
 constexpr int MAXG = 8;
 
+// x / d = umulhi(x, mul) >> shr for x < 2^31 (d > 1).
+struct FastDiv {
+  unsigned d, mul;
+  int shr;
+};
+
+// A group of indices, extents > 1 only, adjacent ones merged where their
+// strides allow it.
 struct Grp {
   int n;
-  int dim[MAXG];
+  FastDiv dim[MAXG];
   long long s[MAXG];
 };
 
@@ -150,13 +158,29 @@ __device__ __forceinline__ float round_tf32(float x) {
   return __uint_as_float(r);
 }
 
+__device__ __forceinline__ unsigned fast_div(unsigned x, const FastDiv& f) {
+  return f.d > 1 ? __umulhi(x, f.mul) >> f.shr : x;
+}
+
+// Offset of index idx < 2^31 of a group: 32-bit divisions by precomputed
+// reciprocals (64-bit ones took ~1 us of a small launch).
 __device__ __forceinline__ void decomp(const Grp& g, long long idx, long long& off) {
   off = 0;
-  for (int i = g.n - 1; i >= 0; --i) {
-    const long long q = idx / g.dim[i];
-    off += (idx - q * g.dim[i]) * g.s[i];
-    idx = q;
+  unsigned x = unsigned(idx);
+  for (int i = g.n - 1; i > 0; --i) {
+    const unsigned q = fast_div(x, g.dim[i]);
+    off += (x - q * g.dim[i].d) * g.s[i];
+    x = q;
   }
+  if (g.n > 0) off += x * g.s[0];
+}
+
+// double(v) by bits: the conversion instruction holds the FP64 pipe of an SM
+// quarter for 64 clocks a warp.
+__device__ __forceinline__ double widen(float v) {
+  const unsigned u = __float_as_uint(v), e = (u >> 23) & 0xff;
+  if (e == 0 || e == 255) return double(v);
+  return __hiloint2double(int((u & 0x80000000u) | (((u >> 3) & 0x0fffffffu) + (896u << 20))), int(u << 29));
 }
 
 // Element o of problem pb's output: FP64, FP32, or a tensor-core operand of
@@ -165,7 +189,7 @@ __device__ __forceinline__ void decomp(const Grp& g, long long idx, long long& o
 // from the FP32 result.
 __device__ __forceinline__ void put_out(const TcArgs& g, int pb, long long o, float v) {
   if (g.out_f64) {
-    static_cast<double*>(g.C.p[pb])[o] = double(v);
+    static_cast<double*>(g.C.p[pb])[o] = widen(v);
   } else if (g.out_tc == 2) {
     const __nv_bfloat16 h = __float2bfloat16(v);
     static_cast<__nv_bfloat16*>(g.C.p[pb])[o] = h;
@@ -185,7 +209,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const __grid_constant__ 
                                                         const __grid_constant__ CUtensorMap tb,
                                                         const __grid_constant__ CUtensorMap tal,
                                                         const __grid_constant__ CUtensorMap tbl,
-                                                        const TcArgs g) {
+                                                        const __grid_constant__ TcArgs g) {
   constexpr int A_BYTES = TC_BM * TC_ROWB;
   constexpr int B_BYTES = BN * TC_ROWB;
   extern __shared__ __align__(1024) uint8_t dsm[];
@@ -377,7 +401,7 @@ __global__ void __launch_bounds__(TCP_THREADS) k_gemm_tc_persist(const __grid_co
                                                                  const __grid_constant__ CUtensorMap tb,
                                                                  const __grid_constant__ CUtensorMap tal,
                                                                  const __grid_constant__ CUtensorMap tbl,
-                                                                 const TcArgs g) {
+                                                                 const __grid_constant__ TcArgs g) {
   constexpr int A_BYTES = TC_BM * TC_ROWB;
   constexpr int B_BYTES = BN * TC_ROWB;
   constexpr int NCOL = BN < 32 ? 32 : BN;   // TMEM columns of one accumulator
@@ -569,16 +593,27 @@ __global__ void __launch_bounds__(TCP_THREADS) k_gemm_tc_persist(const __grid_co
 
 // Split-K: out[p][m, n] = alpha * sum_s part[s][p][m][n] (fixed order), through
 // the output offset groups.
-__global__ void k_tc_splitk_reduce(const TcArgs g) {
-  const long long MN = g.M * g.N, total = (long long)g.nprob * MN;
+__global__ void __launch_bounds__(256) k_tc_splitk_reduce(const __grid_constant__ TcArgs g, FastDiv by_n) {
+  const long long MN = g.M * g.N;
+  const int pb = blockIdx.y;
   const float alpha = float(g.alpha);
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int pb = int(t / MN);
-    const long long mn = t - pb * MN, m = mn / g.N, n = mn - m * g.N;
+  for (long long mn = blockIdx.x * (long long)blockDim.x + threadIdx.x; mn < MN;
+       mn += (long long)gridDim.x * blockDim.x) {
+    const float* part = g.part + pb * MN + mn;
+    const long long step = g.nprob * MN;
     float v = 0.f;
-    for (int sp = 0; sp < g.splitk; ++sp) v += g.part[((long long)sp * g.nprob + pb) * MN + mn];
+#pragma unroll 8
+    for (int sp = 0; sp < g.splitk; ++sp) v += part[sp * step];
     v *= alpha;
+    long long m, n;
+    if (MN < (1LL << 31)) {
+      const unsigned q = fast_div(unsigned(mn), by_n);
+      m = q;
+      n = unsigned(mn) - q * by_n.d;
+    } else {
+      m = mn / g.N;
+      n = mn - m * g.N;
+    }
     long long om, on;
     decomp(g.gm, m, om);
     decomp(g.gn, n, on);
@@ -589,8 +624,8 @@ __global__ void k_tc_splitk_reduce(const TcArgs g) {
 // Gather-copy into a dense [rows][ld] operand: element (r, k) of the output is
 // src[sum(idx_i * stride_i)] with r, k decomposed over the row / K groups.
 // Rounds to TF32 (or converts to BF16); `lo` receives the rounded residual.
-// Tiled transpose: each CTA moves a 64 x 64 (row, k) tile through shared
-// memory, decomposing its 64 row and 64 k offsets once; reads run along
+// Tiled transpose: each CTA moves a square (row, k) tile through shared
+// memory, decomposing its row and k offsets once; reads run along
 // whichever group holds the source's unit stride (rows_fast), writes run along
 // k, so both sides are coalesced whatever the permutation.
 struct PackArgs {
@@ -607,8 +642,9 @@ struct PackArgs {
 // 64 x 64 (row, k) tiles, 256 threads, 16 elements per thread: the offsets
 // of a tile's 64 rows and 64 k are decomposed once (128 threads), then every
 // thread issues all 16 of its loads before it stores, so each warp keeps 16
-// coalesced loads in flight.
-constexpr int PK_T = 64;
+// coalesced loads in flight.  32 x 32 tiles where 64 x 64 ones would be fewer
+// than the SMs: the rounding of an element is ~60 instructions, so a small
+// operand takes as long as one CTA's share of it.
 
 // hi = v rounded to the operand type; lo = the rounded residual.  For FP32
 // sources everything stays in FP32 (v - tf32(v) is exact there): the FP64
@@ -624,7 +660,13 @@ __device__ __forceinline__ void split_store(float v, const PackArgs& p, long lon
     if (p.lo) static_cast<float*>(p.lo)[d] = round_tf32(v - h);
   }
 }
-__device__ __forceinline__ void split_store(double v, const PackArgs& p, long long d) {
+// The same values for FP64 sources, rounded on the bits: v is an integer
+// mv = (1, mantissa) times 2^(ex - 52); h takes its leading bits, rounded to
+// nearest even (for TF32 through FP32 first, as the conversions do), and the
+// residual is the exact integer mv - mh.  Conversions and an FP64 subtraction
+// cost 3 to 5 passes of the FP64 pipe per element, several times the copy.
+// Values whose parts leave FP32's normal range take the plain conversions.
+__device__ __forceinline__ void split_plain(double v, const PackArgs& p, long long d) {
   if (p.bf16) {
     const __nv_bfloat16 h = __double2bfloat16(v);
     static_cast<__nv_bfloat16*>(p.hi)[d] = h;
@@ -636,15 +678,71 @@ __device__ __forceinline__ void split_store(double v, const PackArgs& p, long lo
   }
 }
 
+// x / 2^n rounded to nearest even, 0 < n < 64.
+__device__ __forceinline__ unsigned long long shift_rne(unsigned long long x, int n) {
+  const unsigned long long q = x >> n, rem = x & ((1ULL << n) - 1), half = 1ULL << (n - 1);
+  return q + (rem > half || (rem == half && (q & 1)) ? 1 : 0);
+}
+
+// FP32 bits of (sign, m 2^ex) with m rounded to `bits` significant bits
+// (nearest even); m > 0, the result in FP32's normal range.
+__device__ __forceinline__ unsigned round_bits(unsigned sign, unsigned long long m, int ex, int bits) {
+  const int len = 64 - __clzll((long long)m);
+  unsigned long long r = m;
+  int e = ex;
+  if (len > bits) {
+    r = shift_rne(m, len - bits);
+    e += len - bits;
+    if (r >> bits) {   // rounded up to 2^bits
+      r >>= 1;
+      ++e;
+    }
+  }
+  const int rl = 64 - __clzll((long long)r);
+  const unsigned frac = unsigned(r << (24 - rl)) & 0x7fffffu;
+  return sign | (unsigned(e + rl - 1 + 127) << 23) | frac;
+}
+
+__device__ __forceinline__ void split_store(double v, const PackArgs& p, long long d) {
+  const unsigned hi = unsigned(__double2hiint(v));
+  const int ex = int((hi >> 20) & 0x7ff) - 1023;
+  if (ex < -60 || ex > 100) {
+    split_plain(v, p, d);   // zeros too
+    return;
+  }
+  const unsigned sign = hi & 0x80000000u;
+  const unsigned long long mv =
+      ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | unsigned(__double2loint(v));
+  // h as FP32 bits: BF16 has 8 significant bits, TF32 11 after FP32's 24
+  unsigned hb;
+  if (p.bf16)
+    hb = round_bits(sign, mv, ex - 52, 8);
+  else
+    hb = __float_as_uint(round_tf32(__uint_as_float(round_bits(sign, mv, ex - 52, 24))));
+  const int he = int((hb >> 23) & 0xff) - 127;
+  const long long mh = (long long)((hb & 0x7fffffu) | 0x800000u) << (29 + he - ex);
+  const long long r = (long long)mv - mh;   // |v| - |h| in units of 2^(ex - 52)
+  unsigned lb = 0;
+  if (r != 0) lb = round_bits(r < 0 ? sign ^ 0x80000000u : sign, (unsigned long long)(r < 0 ? -r : r), ex - 52, p.bf16 ? 8 : 24);
+  if (p.bf16) {
+    static_cast<unsigned short*>(p.hi)[d] = (unsigned short)(hb >> 16);
+    if (p.lo) static_cast<unsigned short*>(p.lo)[d] = (unsigned short)(lb >> 16);
+  } else {
+    static_cast<float*>(p.hi)[d] = __uint_as_float(hb);
+    if (p.lo) static_cast<float*>(p.lo)[d] = round_tf32(__uint_as_float(lb));
+  }
+}
+
 // Grid = (row tiles x k tiles, problems), 256 threads; T = source element type.
-template <typename T>
-__global__ void __launch_bounds__(256) k_pack(const PackArgs p) {
+template <typename T, int PK_T>
+__global__ void __launch_bounds__(256) k_pack(const __grid_constant__ PackArgs p) {
   __shared__ T tile[PK_T][PK_T + 1];   // [k][row]
   __shared__ long long ro[PK_T], ko[PK_T];
   const int pb = blockIdx.y;
   const long long ktiles = (p.K + PK_T - 1) / PK_T;
   const long long r0 = (blockIdx.x / ktiles) * PK_T, k0 = (blockIdx.x % ktiles) * PK_T;
-  const int tid = threadIdx.x, tx = tid & (PK_T - 1), ty = tid / PK_T;   // ty in 0..3
+  constexpr int TY = 256 / PK_T;
+  const int tid = threadIdx.x, tx = tid & (PK_T - 1), ty = tid / PK_T;   // ty in 0..TY-1
   if (tid < PK_T) {
     long long o = -1;
     if (r0 + tid < p.rows) decomp(p.gr, r0 + tid, o);
@@ -656,25 +754,25 @@ __global__ void __launch_bounds__(256) k_pack(const PackArgs p) {
   }
   __syncthreads();
   const T* src = static_cast<const T*>(p.src.p[pb]);
-  constexpr int NQ = PK_T / 4;   // 16 elements per thread
+  constexpr int NQ = PK_T / TY;   // elements per thread: 16, or 4
   T v[NQ];
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
-    const int a = ty + 4 * q;
+    const int a = ty + TY * q;
     const int r = p.rows_fast ? tx : a, k = p.rows_fast ? a : tx;
     const long long orr = ro[r], okk = ko[k];
     v[q] = (orr >= 0 && okk >= 0) ? src[orr + okk] : T(0);
   }
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
-    const int a = ty + 4 * q;
+    const int a = ty + TY * q;
     const int r = p.rows_fast ? tx : a, k = p.rows_fast ? a : tx;
     tile[k][r] = v[q];
   }
   __syncthreads();
 #pragma unroll 4
   for (int q = 0; q < NQ; ++q) {
-    const int r = ty + 4 * q, k = tx;
+    const int r = ty + TY * q, k = tx;
     if (ro[r] < 0 || ko[k] < 0) continue;
     split_store(tile[k][r], p, (pb * p.pad + r0 + r) * p.ld + k0 + k);
   }
@@ -741,17 +839,28 @@ std::vector<long long> strides_of(const Dims& d) {
   return s;
 }
 
-void push(Grp& g, int dim, long long s) {
-  PEPS_REQUIRE(g.n < MAXG, "too many indices in one group");
-  g.dim[g.n] = dim;
-  g.s[g.n] = s;
-  g.n++;
+FastDiv fast_divisor(long long d) {
+  FastDiv f{unsigned(d), 0, 0};
+  if (d > 1) {
+    int l = 1;   // ceil(log2 d)
+    while ((1LL << l) < d) ++l;
+    f.mul = unsigned(((1ULL << (31 + l)) + (unsigned long long)d - 1) / (unsigned long long)d);
+    f.shr = l - 1;
+  }
+  return f;
 }
 
-long long prod(const Grp& g) {
-  long long n = 1;
-  for (int i = 0; i < g.n; ++i) n *= g.dim[i];
-  return n;
+void push(Grp& g, int dim, long long s) {
+  if (dim <= 1) return;
+  if (g.n > 0 && g.s[g.n - 1] == s * dim && (long long)g.dim[g.n - 1].d * dim < (1LL << 31)) {
+    g.dim[g.n - 1] = fast_divisor((long long)g.dim[g.n - 1].d * dim);
+    g.s[g.n - 1] = s;
+    return;
+  }
+  PEPS_REQUIRE(g.n < MAXG, "too many indices in one group");
+  g.dim[g.n] = fast_divisor(dim);
+  g.s[g.n] = s;
+  g.n++;
 }
 
 struct Operand {
@@ -768,17 +877,19 @@ Operand pack(Ctx& cx, const TP& src, int np, long long pad, int src_f64, const s
   auto st = strides_of(dims);
   PackArgs p;
   std::memset(static_cast<void*>(&p), 0, sizeof(p));
+  Operand o;
+  o.rows = o.K = 1;
   for (char ch : rowletters) {
     auto i = letters.find(ch);
     push(p.gr, dims[i], st[i]);
+    o.rows *= dims[i];
   }
   for (char ch : kletters) {
     auto i = letters.find(ch);
     push(p.gk, dims[i], st[i]);
+    o.K *= dims[i];
   }
-  Operand o;
-  o.rows = prod(p.gr);
-  o.K = prod(p.gk);
+  PEPS_REQUIRE(o.rows < (1LL << 31) && o.K < (1LL << 31), "operand too large to pack");
   const int align = bf16 ? 8 : 4;
   o.ld = (o.K + align - 1) / align * align;
   PEPS_REQUIRE(pad >= o.rows, "internal: pack padding");
@@ -798,20 +909,29 @@ Operand pack(Ctx& cx, const TP& src, int np, long long pad, int src_f64, const s
   // read along whichever group holds the smaller innermost stride
   auto inner = [](const Grp& g) {
     long long m = 1LL << 62;
-    for (int i = 0; i < g.n; ++i)
-      if (g.dim[i] > 1) m = std::min(m, g.s[i]);
+    for (int i = 0; i < g.n; ++i) m = std::min(m, g.s[i]);
     return m;
   };
   p.rows_fast = inner(p.gr) < inner(p.gk) ? 1 : 0;
-  const long long tiles = ((o.rows + PK_T - 1) / PK_T) * ((o.K + PK_T - 1) / PK_T);
+  auto tiles_of = [&](long long t) { return ((o.rows + t - 1) / t) * ((o.K + t - 1) / t); };
+  const bool small = tiles_of(64) * np < 152;
+  const long long tiles = tiles_of(small ? 32 : 64);
   PEPS_REQUIRE(tiles < (1LL << 31), "operand too large to pack");
   const double moved = double(np) * double(o.rows) * double(o.K) *
                        ((src_f64 ? 8.0 : 4.0) + (split ? 2.0 : 1.0) * (bf16 ? 2.0 : 4.0));
   Launch L(K_PACK, cx.st, 0, moved);
-  if (src_f64)
-    k_pack<double><<<dim3(unsigned(tiles), np), 256, 0, cx.st>>>(p);
-  else
-    k_pack<float><<<dim3(unsigned(tiles), np), 256, 0, cx.st>>>(p);
+  const dim3 grid(unsigned(tiles), np);
+  if (src_f64) {
+    if (small)
+      k_pack<double, 32><<<grid, 256, 0, cx.st>>>(p);
+    else
+      k_pack<double, 64><<<grid, 256, 0, cx.st>>>(p);
+  } else {
+    if (small)
+      k_pack<float, 32><<<grid, 256, 0, cx.st>>>(p);
+    else
+      k_pack<float, 64><<<grid, 256, 0, cx.st>>>(p);
+  }
   PEPS_CHECK_LAUNCH();
   return o;
 }
@@ -1091,15 +1211,14 @@ void ein_tc(Ctx& cx, const char* spec, const TP& A, int a_f64, const Dims& ad, c
     // first tile; on a tie, the one along the smaller innermost stride.
     auto inner = [](const Grp& q) {
       long long m = 1LL << 62;
-      for (int i = 0; i < q.n; ++i)
-        if (q.dim[i] > 1) m = std::min(m, q.s[i]);
+      for (int i = 0; i < q.n; ++i) m = std::min(m, q.s[i]);
       return m;
     };
     auto offset = [](const Grp& q, long long idx) {
       long long o = 0;
       for (int i = q.n - 1; i >= 0; --i) {
-        o += (idx % q.dim[i]) * q.s[i];
-        idx /= q.dim[i];
+        o += (idx % q.dim[i].d) * q.s[i];
+        idx /= q.dim[i].d;
       }
       return o;
     };
@@ -1134,9 +1253,8 @@ void ein_tc(Ctx& cx, const char* spec, const TP& A, int a_f64, const Dims& ad, c
     default: launch_tc<128>(cx, ta, tb, tal, tbl, g, tiles); break;
   }
   if (g.splitk > 1) {
-    const long long total = (long long)np * M * N;
-    const unsigned blocks = unsigned(std::max<long long>(1, std::min<long long>((total + 255) / 256, 4096)));
-    k_tc_splitk_reduce<<<blocks, 256, 0, cx.st>>>(g);
+    const unsigned blocks = unsigned(std::max<long long>(1, std::min<long long>((M * N + 255) / 256, 4096)));
+    k_tc_splitk_reduce<<<dim3(blocks, np), 256, 0, cx.st>>>(g, fast_divisor(N));
     PEPS_CHECK_LAUNCH();
     L.more();
   }
