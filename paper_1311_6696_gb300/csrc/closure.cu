@@ -6,9 +6,12 @@
 // X X^T / ||X X^T||_F, which is positive and equals sigma0 when the network
 // outputs zero.  Labels are the site matrices of the best product (D'=1)
 // approximation of the full boundary at the same cut.  The three GEMMs of
-// each pass run on the tensor cores (BF16 operands, FP32 accumulation);
-// bias, ReLU, the sigma map with its loss and gradient, and AdamW are
-// elementwise kernels here.
+// each pass run on the tensor cores (BF16 operands, FP32 accumulation), with
+// bias, ReLU and the rectifier's mask in their epilogues and every activation
+// written once, as the next layer's BF16 operand; the sigma map with its loss
+// and gradient, the bias gradients and AdamW are kernels here.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 #include <numeric>
@@ -16,6 +19,8 @@
 
 #include "closure.cuh"
 #include "linalg.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace peps {
 namespace {
@@ -183,79 +188,131 @@ __global__ void k_init(float* w, int F, int W, int out, unsigned long long seed)
   }
 }
 
-__global__ void k_bias_act(float* Z, const float* b, long long n, int W, int relu) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n * W; i += (long long)gridDim.x * blockDim.x) {
-    float v = Z[i] + b[i % W];
-    Z[i] = relu ? fmaxf(v, 0.f) : v;
+// Column sums in double of up to three [n][W] matrices in one launch: 8 columns
+// (one 32-byte sector a row) per cluster of 4 CTAs, each a quarter of the rows,
+// added through distributed shared memory in rank order.
+struct ColSums {
+  const float* z[3];
+  float* out[3];
+  int W[3];
+  int blocks[3];   // clusters of each job
+};
+
+__global__ void __launch_bounds__(256) k_colsum(const ColSums s, long long n) {
+  __shared__ double red[8][9], mine[8];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = int(cluster.num_blocks()), rank = int(cluster.block_rank());
+  int b = blockIdx.x / C, job = 0;
+  while (b >= s.blocks[job]) b -= s.blocks[job++];
+  const int W = s.W[job], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = b * 8 + (lane & 7);
+  const long long per = (n + C - 1) / C, r1 = min(n, (rank + 1) * per);
+  double v = 0.0;
+  if (c < W)
+#pragma unroll 4
+    for (long long r = rank * per + warp * 4 + (lane >> 3); r < r1; r += 32) v += s.z[job][r * W + c];
+  v += __shfl_xor_sync(0xffffffffu, v, 8);
+  v += __shfl_xor_sync(0xffffffffu, v, 16);
+  if (lane < 8) red[warp][lane] = v;
+  __syncthreads();
+  if (threadIdx.x < 8) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+    mine[threadIdx.x] = t;
   }
-}
-
-__global__ void k_relu_bwd(float* dH, const float* H, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    if (H[i] <= 0.f) dH[i] = 0.f;
-}
-
-// db[c] = sum_b dZ[b][c]: one block per column chunk, rows strided, fixed order
-__global__ void k_colsum(const float* dZ, long long n, int W, float* db) {
-  __shared__ double red[32];
-  for (int c = blockIdx.x; c < W; c += gridDim.x) {
-    double s = 0.0;
-    for (long long b = threadIdx.x; b < n; b += blockDim.x) s += dZ[b * W + c];
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) db[c] = float(s);
+  cluster.sync();
+  if (rank == 0 && threadIdx.x < 8 && c < W) {
+    double t = 0.0;
+    for (int q = 0; q < C; ++q) t += *cluster.map_shared_rank(mine + threadIdx.x, q);
+    s.out[job][c] = float(t);
   }
+  cluster.sync();
 }
 
-// sigma = X X^T / ||X X^T||, X = L0 + Yo;  loss and dL/dYo (mean over n)
-__global__ void k_sigma(const float* Xin, int F, const float* Yo, const float* lab, long long n, int D, float* sig,
-                        float* dYo, double* loss_part) {
-  __shared__ double red[32];
+// sigma = X X^T / ||X X^T||, X = L0 + Yo, one thread per example.
+__global__ void k_sigma(const float* Xin, int F, const float* Yo, long long n, int D, float* sig) {
   const int DD = D * D;
-  double lsum = 0.0;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     double X[64], S[64];
     const float* L0 = Xin + e * F + (F - DD);
     for (int i = 0; i < DD; ++i) X[i] = double(L0[i]) + double(Yo[e * DD + i]);
     double nr = 0.0;
     for (int i = 0; i < D; ++i)
-      for (int j = 0; j < D; ++j) {
+      for (int j = 0; j <= i; ++j) {
         double a = 0.0;
-        for (int k = 0; k < D; ++k) a += X[i * D + k] * X[j * D + k];
+        for (int k = 0; k < D; ++k) a = fma(X[i * D + k], X[j * D + k], a);
         S[i * D + j] = a;
-        nr += a * a;
+        nr = fma(i == j ? a : 2.0 * a, a, nr);
       }
-    nr = sqrt(nr);
-    const double inv = nr > 0 ? 1.0 / nr : 0.0;
-    if (sig)
-      for (int i = 0; i < DD; ++i) sig[e * DD + i] = float(S[i] * inv);
-    if (lab) {
-      double G[64], gs = 0.0;
-      for (int i = 0; i < DD; ++i) {
-        const double df = S[i] * inv - double(lab[e * DD + i]);
-        lsum += df * df;
-        G[i] = 2.0 * df / double(n);
-        gs += G[i] * S[i] * inv;
-      }
-      double dS[64];
-      for (int i = 0; i < DD; ++i) dS[i] = (G[i] - S[i] * inv * gs) * inv;
-      for (int i = 0; i < D; ++i)
-        for (int k = 0; k < D; ++k) {
-          double a = 0.0;
-          for (int j = 0; j < D; ++j) a += (dS[i * D + j] + dS[j * D + i]) * X[j * D + k];
-          dYo[e * DD + i * D + k] = float(a);
-        }
-    }
-  }
-  if (loss_part) {
-    lsum = block_sum(lsum, red);
-    if (threadIdx.x == 0) loss_part[blockIdx.x] = lsum;
+    const double inv = nr > 0 ? 1.0 / sqrt(nr) : 0.0;
+    for (int i = 0; i < D; ++i)
+      for (int j = 0; j < D; ++j) sig[e * DD + i * D + j] = float(S[i > j ? i * D + j : j * D + i] * inv);
   }
 }
 
+// Sum over a group of G lanes (a power of two), in every lane.
+__device__ __forceinline__ double group_sum(double v, int G) {
+  for (int o = G >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Loss and dL/dYo (mean over n).  G lanes per example, an entry (i, k) of the
+// D x D matrices each (two above 32): the chain of one thread per example --
+// ~600 FP64 instructions of 64 clocks -- took 45 us whatever n was.
+__global__ void __launch_bounds__(256) k_sigma_grad(const float* Xin, int F, const float* Yo, const float* lab,
+                                                    long long n, int D, int G, float* dYo, double* loss_part) {
+  __shared__ double red[32];
+  __shared__ double xs[8][64], ss[8][64];   // per warp: X and dS of its 32 / G examples
+  const int DD = D * D, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, per = 32 / G, l = lane & (G - 1);
+  const int slot = (lane / G) * DD;
+  double* X = xs[warp] + slot;
+  double* dS = ss[warp] + slot;
+  const double two_n = 2.0 / double(n);
+  double lsum = 0.0;
+  for (long long e0 = (blockIdx.x * 8LL + warp) * per; e0 < n; e0 += gridDim.x * 8LL * per) {
+    const long long e = e0 + lane / G;
+    const bool in = e < n;
+    for (int t = l; t < DD; t += G) X[t] = in ? double(Xin[e * F + (F - DD) + t]) + double(Yo[e * DD + t]) : 0.0;
+    __syncwarp();
+    double S[2] = {0.0, 0.0}, nr = 0.0;
+    for (int t = l, u = 0; t < DD; t += G, ++u) {
+      const int i = t / D, j = t - i * D;
+      double a = 0.0;
+      for (int k = 0; k < D; ++k) a = fma(X[i * D + k], X[j * D + k], a);
+      S[u] = a;
+      nr = fma(a, a, nr);
+    }
+    nr = group_sum(nr, G);
+    const double inv = nr > 0 ? 1.0 / sqrt(nr) : 0.0;
+    double g[2] = {0.0, 0.0}, gs = 0.0;
+    for (int t = l, u = 0; t < DD; t += G, ++u) {
+      S[u] *= inv;
+      const double df = in ? S[u] - double(lab[e * DD + t]) : 0.0;
+      lsum = fma(df, df, lsum);
+      g[u] = two_n * df;
+      gs = fma(g[u], S[u], gs);
+    }
+    gs = group_sum(gs, G);
+    for (int t = l, u = 0; t < DD; t += G, ++u) dS[t] = (g[u] - S[u] * gs) * inv;
+    __syncwarp();
+    for (int t = l; t < DD; t += G) {
+      const int i = t / D, k = t - i * D;
+      double a = 0.0;
+      for (int j = 0; j < D; ++j) a = fma(dS[i * D + j] + dS[j * D + i], X[j * D + k], a);
+      if (in) dYo[e * DD + t] = float(a);
+    }
+    __syncwarp();
+  }
+  lsum = block_sum(lsum, red);
+  if (threadIdx.x == 0) loss_part[blockIdx.x] = lsum;
+}
+
 __global__ void k_sum_loss(const double* part, int np, long long n, double* out, int accumulate) {
-  if (threadIdx.x || blockIdx.x) return;
+  __shared__ double red[32];
   double s = 0.0;
-  for (int i = 0; i < np; ++i) s += part[i];
+  for (int i = threadIdx.x; i < np; i += blockDim.x) s += part[i];
+  s = block_sum(s, red);
+  if (threadIdx.x) return;
   s /= double(n);
   out[0] = accumulate ? out[0] + s : s;
 }
@@ -294,6 +351,12 @@ __global__ void k_apply(const float* pred, double* const* targets, long long n, 
   for (int i = 0; i < DD; ++i) targets[e][i] = double(pred[e * DD + i]);
 }
 
+// Blocks of k_sigma_grad: 8 warps, 32 / G examples each.
+unsigned loss_blocks(long long n, int G) {
+  const long long per = 8 * (32 / G);
+  return unsigned(std::max<long long>(1, std::min<long long>((n + per - 1) / per, 4096)));
+}
+
 unsigned grid_for(long long n) {
   return unsigned(std::max<long long>(1, std::min<long long>((n + 255) / 256, 4096)));
 }
@@ -316,25 +379,41 @@ Layers layers(const MlpDims& m, const float* w) {
 
 constexpr int kMlpPrec = PEPS_PREC_BF16;
 
-// Forward pass; H1, H2 (n x W) and Yo (n x out) are caller buffers.
-void forward(Ctx& cx, const MlpDims& m, const float* w, const float* X, long long n, float* H1, float* H2, float* Yo) {
+// Activations H1, H2 of a forward pass: BF16 [n][W] in the layout of the next
+// layer's operand, biased, rectified and rounded by the GEMM that makes them
+// (the values an operand pack of the FP32 activations would make).
+size_t act_words(const MlpDims& m, long long n) {
+  return tc_operand_words("bw,vw->bv", {int(n), m.W}, {m.W, m.W}, 1, kMlpPrec);
+}
+
+// Forward pass; H1, H2 (act_words each) and Yo (n x out) are caller buffers.
+void forward(Ctx& cx, const MlpDims& m, const float* w, const float* X, long long n, double* H1, double* H2, float* Yo) {
   const Layers L = layers(m, w);
   const int F = m.F(), W = m.W, o = m.out();
   const int nn = int(n);
-  ein_tc(cx, "bi,wi->bw", X, 0, {nn, F}, L.W1, 0, {W, F}, H1, 0, kMlpPrec);
-  {
-    Launch l(K_AUX, cx.st);
-    k_bias_act<<<grid_for(n * W), 256, 0, cx.st>>>(H1, L.b1, n, W, 1);
-  }
-  ein_tc(cx, "bw,vw->bv", H1, 0, {nn, W}, L.W2, 0, {W, W}, H2, 0, kMlpPrec);
-  {
-    Launch l(K_AUX, cx.st);
-    k_bias_act<<<grid_for(n * W), 256, 0, cx.st>>>(H2, L.b2, n, W, 1);
-  }
-  ein_tc(cx, "bv,ov->bo", H2, 0, {nn, W}, L.W3, 0, {o, W}, Yo, 0, kMlpPrec);
-  Launch l(K_AUX, cx.st);
-  k_bias_act<<<grid_for(n * o), 256, 0, cx.st>>>(Yo, L.b3, n, o, 0);
-  PEPS_CHECK_LAUNCH();
+  const size_t cap = act_words(m, n);
+  TcOperand o1, o2;
+  TcChain c1, c2, c3;
+  c1.next = "bw,vw->bv";
+  c1.next_bd = {W, W};
+  c1.next_mem = H1;
+  c1.next_cap = cap;
+  c1.next_out = &o1;
+  c1.bias = L.b1;
+  c1.relu = true;
+  ein_tc(cx, "bi,wi->bw", X, 0, {nn, F}, L.W1, 0, {W, F}, TP(), 0, kMlpPrec, 1.0, TP(), nullptr, &c1);
+  c2.a_pre = &o1;
+  c2.next = "bv,ov->bo";
+  c2.next_bd = {o, W};
+  c2.next_mem = H2;
+  c2.next_cap = cap;
+  c2.next_out = &o2;
+  c2.bias = L.b2;
+  c2.relu = true;
+  ein_tc(cx, "bw,vw->bv", TP(), 0, {nn, W}, L.W2, 0, {W, W}, TP(), 0, kMlpPrec, 1.0, TP(), nullptr, &c2);
+  c3.a_pre = &o2;
+  c3.bias = L.b3;
+  ein_tc(cx, "bv,ov->bo", TP(), 0, {nn, W}, L.W3, 0, {o, W}, Yo, 0, kMlpPrec, 1.0, TP(), nullptr, &c3);
 }
 
 }  // namespace
@@ -367,12 +446,12 @@ void mlp_init(Ctx& cx, const MlpDims& m, float* w, unsigned long long seed) {
 
 void mlp_predict(Ctx& cx, const MlpDims& m, const float* w, const float* X, long long n, float* sigma) {
   if (n == 0) return;
-  float* H1 = cx.ws->falloc(size_t(n) * m.W);
-  float* H2 = cx.ws->falloc(size_t(n) * m.W);
+  double* H1 = cx.ws->dalloc(act_words(m, n));
+  double* H2 = cx.ws->dalloc(act_words(m, n));
   float* Yo = cx.ws->falloc(size_t(n) * m.out());
   forward(cx, m, w, X, n, H1, H2, Yo);
   Launch l(K_AUX, cx.st);
-  k_sigma<<<grid_for(n), 256, 0, cx.st>>>(X, m.F(), Yo, nullptr, n, m.D, sigma, nullptr, nullptr);
+  k_sigma<<<unsigned(std::min<long long>((n + 63) / 64, 4096)), 64, 0, cx.st>>>(X, m.F(), Yo, n, m.D, sigma);
   PEPS_CHECK_LAUNCH();
 }
 
@@ -380,16 +459,18 @@ namespace {
 // Loss (accumulated into loss_dev if accumulate) and gradient for n examples,
 // with caller-provided activation buffers.
 void loss_grad_buf(Ctx& cx, const MlpDims& m, const float* w, const float* X, const float* Y, long long n,
-                   double* loss_dev, int accumulate, float* grad, float* H1, float* H2, float* Yo, float* dYo,
+                   double* loss_dev, int accumulate, float* grad, double* H1, double* H2, float* Yo, float* dYo,
                    float* dH1, float* dH2, double* part) {
   const Layers L = layers(m, w);
   const int F = m.F(), W = m.W, o = m.out(), nn = int(n);
   forward(cx, m, w, X, n, H1, H2, Yo);
-  const unsigned gs = grid_for(n);
+  int G = 4;   // lanes per example of the loss
+  while (G < o && G < 32) G *= 2;
+  const unsigned gs = loss_blocks(n, G);
   {
     Launch l(K_AUX, cx.st);
-    k_sigma<<<gs, 256, 0, cx.st>>>(X, F, Yo, Y, n, m.D, nullptr, dYo, part);
-    k_sum_loss<<<1, 32, 0, cx.st>>>(part, int(gs), n, loss_dev, accumulate);
+    k_sigma_grad<<<gs, 256, 0, cx.st>>>(X, F, Yo, Y, n, m.D, G, dYo, part);
+    k_sum_loss<<<1, 256, 0, cx.st>>>(part, int(gs), n, loss_dev, accumulate);
     PEPS_CHECK_LAUNCH();
     l.more();
   }
@@ -399,26 +480,43 @@ void loss_grad_buf(Ctx& cx, const MlpDims& m, const float* w, const float* X, co
   float* gb2 = gW2 + (long long)W * W;
   float* gW3 = gb2 + W;
   float* gb3 = gW3 + (long long)o * W;
-  ein_tc(cx, "bo,bv->ov", dYo, 0, {nn, o}, H2, 0, {nn, W}, gW3, 0, kMlpPrec);
-  ein_tc(cx, "bo,ov->bv", dYo, 0, {nn, o}, L.W3, 0, {o, W}, dH2, 0, kMlpPrec);
-  {
-    Launch l(K_AUX, cx.st);
-    k_colsum<<<std::min(o, 1024), 256, 0, cx.st>>>(dYo, n, o, gb3);
-    k_relu_bwd<<<grid_for(n * W), 256, 0, cx.st>>>(dH2, H2, n * W);
-    k_colsum<<<std::min(W, 1024), 256, 0, cx.st>>>(dH2, n, W, gb2);
-    PEPS_CHECK_LAUNCH();
-    l.more(2);
-  }
-  ein_tc(cx, "bv,bw->vw", dH2, 0, {nn, W}, H1, 0, {nn, W}, gW2, 0, kMlpPrec);
-  ein_tc(cx, "bv,vw->bw", dH2, 0, {nn, W}, L.W2, 0, {W, W}, dH1, 0, kMlpPrec);
-  {
-    Launch l(K_AUX, cx.st);
-    k_relu_bwd<<<grid_for(n * W), 256, 0, cx.st>>>(dH1, H1, n * W);
-    k_colsum<<<std::min(W, 1024), 256, 0, cx.st>>>(dH1, n, W, gb1);
-    PEPS_CHECK_LAUNCH();
-    l.more();
-  }
+  // the activations are BF16 tensors [n][W]; what the rectifier held back is
+  // masked where the gradient is made
+  TcChain m2, m1;
+  m2.mask = H2;
+  m1.mask = H1;
+  ein_tc(cx, "bo,bv->ov", dYo, 0, {nn, o}, H2, 2, {nn, W}, gW3, 0, kMlpPrec);
+  ein_tc(cx, "bo,ov->bv", dYo, 0, {nn, o}, L.W3, 0, {o, W}, dH2, 0, kMlpPrec, 1.0, TP(), nullptr, &m2);
+  ein_tc(cx, "bv,bw->vw", dH2, 0, {nn, W}, H1, 2, {nn, W}, gW2, 0, kMlpPrec);
+  ein_tc(cx, "bv,vw->bw", dH2, 0, {nn, W}, L.W2, 0, {W, W}, dH1, 0, kMlpPrec, 1.0, TP(), nullptr, &m1);
   ein_tc(cx, "bw,bi->wi", dH1, 0, {nn, W}, X, 0, {nn, F}, gW1, 0, kMlpPrec);
+  {
+    ColSums c;
+    c.z[0] = dYo;
+    c.z[1] = dH2;
+    c.z[2] = dH1;
+    c.out[0] = gb3;
+    c.out[1] = gb2;
+    c.out[2] = gb1;
+    c.W[0] = o;
+    c.W[1] = c.W[2] = W;
+    int total = 0;
+    for (int i = 0; i < 3; ++i) total += c.blocks[i] = (c.W[i] + 7) / 8;
+    Launch l(K_AUX, cx.st);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(4 * total, 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = cx.st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 4;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    PEPS_CUDA(cudaLaunchKernelEx(&cfg, k_colsum, c, n));
+    PEPS_CHECK_LAUNCH();
+  }
 }
 }  // namespace
 
@@ -426,13 +524,13 @@ void mlp_loss_grad(Ctx& cx, const MlpDims& m, const float* w, const float* X, co
                    double* loss_dev, float* grad) {
   PEPS_REQUIRE(n > 0, "empty batch");
   const size_t W = m.W, o = m.out();
-  float* H1 = cx.ws->falloc(n * W);
-  float* H2 = cx.ws->falloc(n * W);
+  double* H1 = cx.ws->dalloc(act_words(m, n));
+  double* H2 = cx.ws->dalloc(act_words(m, n));
   float* Yo = cx.ws->falloc(n * o);
   float* dYo = cx.ws->falloc(n * o);
   float* dH1 = cx.ws->falloc(n * W);
   float* dH2 = cx.ws->falloc(n * W);
-  double* part = cx.ws->dalloc(grid_for(n) + 1);
+  double* part = cx.ws->dalloc(4096);
   loss_grad_buf(cx, m, w, X, Y, n, loss_dev, 0, grad, H1, H2, Yo, dYo, dH1, dH2, part);
 }
 
@@ -454,13 +552,13 @@ void mlp_train(Ctx& cx, const MlpDims& m, float* w, const float* X, const float*
   }
   float* Xb = cx.ws->falloc(B * F);
   float* Yb = cx.ws->falloc(B * o);
-  float* H1 = cx.ws->falloc(B * W);
-  float* H2 = cx.ws->falloc(B * W);
+  double* H1 = cx.ws->dalloc(act_words(m, B));
+  double* H2 = cx.ws->dalloc(act_words(m, B));
   float* Yo = cx.ws->falloc(B * o);
   float* dYo = cx.ws->falloc(B * o);
   float* dH1 = cx.ws->falloc(B * W);
   float* dH2 = cx.ws->falloc(B * W);
-  double* part = cx.ws->dalloc(grid_for(B) + 1);
+  double* part = cx.ws->dalloc(4096 + 1);
   double* loss_acc = cx.ws->dalloc(1);
   PEPS_CUDA(cudaMemsetAsync(loss_acc, 0, sizeof(double), cx.st));
   long long* didx = static_cast<long long*>(cx.ws->alloc(sizeof(long long) * size_t(steps) * B));
@@ -498,7 +596,7 @@ void mlp_train(Ctx& cx, const MlpDims& m, float* w, const float* X, const float*
       l.more();
     }
     const bool rec = t >= steps - tail;
-    loss_grad_buf(cx, m, w, Xb, Yb, B, rec ? loss_acc : part + grid_for(B), rec ? 1 : 0, grad, H1, H2, Yo, dYo,
+    loss_grad_buf(cx, m, w, Xb, Yb, B, rec ? loss_acc : part + 4096, rec ? 1 : 0, grad, H1, H2, Yo, dYo,
                   dH1, dH2, part);
     const float c1 = 1.f - std::pow(b1, float(t0 + t + 1)), c2 = 1.f - std::pow(b2, float(t0 + t + 1));
     Launch l(K_AUX, cx.st);

@@ -113,7 +113,7 @@ void ein(Ctx& cx, const char* spec, const TP& A, const Dims& ad, const TP& B,
          const Dims& bd, const TP& C, double alpha = 1.0, double beta = 0.0);
 
 // C = alpha * contract(A, B) on the tensor cores (tcgen05): operands are
-// FP64 (x_f64 = 1) or FP32 tensors, repacked to TF32 / BF16; C is written as
+// FP64 (x_f64 = 1), FP32 or BF16 (x_f64 = 2) tensors, repacked to TF32 / BF16; C is written as
 // FP64 or FP32 in any index order; with Clo (FP32 output only) C receives the
 // TF32-rounded value and Clo the rounded residual.  prec is PEPS_PREC_*.
 // Packed tensor-core copies of B operands that stay unchanged for the cache's
@@ -149,6 +149,9 @@ struct TcOperand {
 //             receives its description.  C and Clo are then ignored.
 // K is ordered as in a plain call, so the result is the same as packing the
 // FP32 output of a plain call.
+//   bias:     added to every row of the result (one value per index of the N
+//             group), before relu (max with 0).
+//   mask:     BF16 tensor [M][N]; results where it is not positive become 0.
 struct TcChain {
   const TcOperand* a_pre = nullptr;
   const char* next = nullptr;
@@ -156,6 +159,9 @@ struct TcChain {
   double* next_mem = nullptr;
   size_t next_cap = 0;
   TcOperand* next_out = nullptr;
+  const float* bias = nullptr;
+  bool relu = false;
+  const void* mask = nullptr;
 };
 
 // Doubles a TcChain target needs for operand A of `spec` (hi and lo parts).

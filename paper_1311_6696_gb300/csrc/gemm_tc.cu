@@ -26,6 +26,7 @@
 #include <mutex>
 #include <cstdlib>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "ein.cuh"
@@ -65,8 +66,10 @@ struct TcArgs {
                      // rounded), 2 = BF16; with out_lo the rounded residual goes to C_lo
   int stages;        // ring depth (<= TC_STAGES), chosen to fit shared memory
   int nprob;         // problems in this launch
-  int cols_fast;     // 1: the output's unit stride is in the N group (write along columns)
+  int cols_fast;     // 1: the output's unit stride is in the N group (write along columns);
+                     // 2: in runs of 16 aligned columns (vector stores)
   int splitk;        // > 1: blockIdx.y takes k tiles [y * kt_per, ...) and writes FP32 partials
+  int parts;         // > 1: the CTA accumulates k tiles [q * kt_per, ...) apart, q < parts, and adds them in order
   int kt_per;
   float* part;       // [splitk][nprob][M][N] partial sums
   long long pad_m, pad_n;   // packed rows per problem (multiples of TC_BM and BN)
@@ -74,7 +77,18 @@ struct TcArgs {
   Grp gm, gn;        // output offsets of the M and N groups
   double alpha;
   int* flag;
+  const float* bias;            // per column, or nullptr
+  const __nv_bfloat16* mask;    // [M][N], or nullptr
+  int relu;
 };
+
+// The result of column n (bias b), row m, from its scaled sum.
+__device__ __forceinline__ float finish_value(const TcArgs& g, long long m, long long n, float b, float v) {
+  v += b;
+  if (g.relu) v = fmaxf(v, 0.f);
+  if (g.mask && __bfloat162float(g.mask[m * g.N + n]) <= 0.f) v = 0.f;
+  return v;
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -203,8 +217,71 @@ __device__ __forceinline__ void put_out(const TcArgs& g, int pb, long long o, fl
   }
 }
 
+// The 16 results at offsets o .. o + 15 (16-byte aligned), the values put_out
+// would write one by one, in 16-byte stores.
+__device__ __forceinline__ void put_run(const TcArgs& g, int pb, long long o, const float* v) {
+  if (g.out_f64) {
+    double2* d = reinterpret_cast<double2*>(static_cast<double*>(g.C.p[pb]) + o);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) d[j] = make_double2(widen(v[2 * j]), widen(v[2 * j + 1]));
+  } else if (g.out_tc == 2) {
+    uint32_t h[8], l[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const __nv_bfloat162 hv = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+      const __nv_bfloat162 lv = __floats2bfloat162_rn(v[2 * j] - __low2float(hv), v[2 * j + 1] - __high2float(hv));
+      h[j] = *reinterpret_cast<const uint32_t*>(&hv);
+      l[j] = *reinterpret_cast<const uint32_t*>(&lv);
+    }
+    uint4* d = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(g.C.p[pb]) + o);
+    d[0] = make_uint4(h[0], h[1], h[2], h[3]);
+    d[1] = make_uint4(h[4], h[5], h[6], h[7]);
+    if (g.out_lo) {
+      uint4* e = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(g.Clo.p[pb]) + o);
+      e[0] = make_uint4(l[0], l[1], l[2], l[3]);
+      e[1] = make_uint4(l[4], l[5], l[6], l[7]);
+    }
+  } else {
+    const bool rounded = g.out_tc == 1 || g.out_lo;
+    float4* d = reinterpret_cast<float4*>(static_cast<float*>(g.C.p[pb]) + o);
+    float4* e = g.out_lo ? reinterpret_cast<float4*>(static_cast<float*>(g.Clo.p[pb]) + o) : nullptr;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float4 x = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+      if (rounded) {
+        const float4 h = make_float4(round_tf32(x.x), round_tf32(x.y), round_tf32(x.z), round_tf32(x.w));
+        if (e) e[j] = make_float4(round_tf32(x.x - h.x), round_tf32(x.y - h.y), round_tf32(x.z - h.z), round_tf32(x.w - h.w));
+        x = h;
+      }
+      d[j] = x;
+    }
+  }
+}
+
+// Bias, rectifier and mask on a lane's 16 scaled results of row m, columns n .. n + 15.
+__device__ __forceinline__ void finish_run(const TcArgs& g, long long m, long long n, const float* bias, float* v) {
+  uint4 mk[2];
+  const bool vec = g.mask && g.N % 16 == 0 && m < g.M && n + 15 < g.N;
+  if (vec) {
+    const uint4* src = reinterpret_cast<const uint4*>(g.mask + m * g.N + n);
+    mk[0] = src[0];
+    mk[1] = src[1];
+  }
+  const __nv_bfloat16* mh = reinterpret_cast<const __nv_bfloat16*>(mk);
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    v[j] += bias[j];
+    if (g.relu) v[j] = fmaxf(v[j], 0.f);
+    if (vec) {
+      if (__bfloat162float(mh[j]) <= 0.f) v[j] = 0.f;
+    } else if (g.mask && m < g.M && n + j < g.N) {
+      if (__bfloat162float(g.mask[m * g.N + n + j]) <= 0.f) v[j] = 0.f;
+    }
+  }
+}
+
 // One 128 x BN output tile per CTA.
-template <int BN>
+template <int BN, bool EX>
 __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const __grid_constant__ CUtensorMap ta,
                                                         const __grid_constant__ CUtensorMap tb,
                                                         const __grid_constant__ CUtensorMap tal,
@@ -219,6 +296,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const __grid_constant__ 
   __shared__ __align__(8) uint64_t full[TC_STAGES], empty[TC_STAGES], done;
   __shared__ uint32_t tmem_base;
   __shared__ long long offm[TC_BM], offn[BN];
+  __shared__ float bias_s[EX ? BN : 1];
   __shared__ float stage_out[4][32][17];   // per warp: 32 rows x 16 columns of the accumulator
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -238,8 +316,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const __grid_constant__ 
     mbar_init(&done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  constexpr uint32_t NCOL = BN < 32 ? 32 : BN;   // TMEM columns of one accumulator
+  const uint32_t ncols = g.parts > 2 ? 4 * NCOL : g.parts > 1 ? 2 * NCOL : NCOL;
   if (warp == 0) {
-    const uint32_t ncols = BN < 32 ? 32 : BN;
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
                  "r"(ncols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -255,6 +334,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const __grid_constant__ 
     long long o = -1;
     if (n < g.N) decomp(g.gn, n, o);
     offn[i] = o;
+    if (EX) bias_s[i] = g.bias && n < g.N ? g.bias[n] : 0.f;
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -296,21 +376,24 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const __grid_constant__ 
       uint8_t* st = base + s * stage_bytes;
       const uint64_t da = sdesc(st), db = sdesc(st + A_BYTES);
       const uint64_t dal = sdesc(st + A_BYTES + B_BYTES), dbl = sdesc(st + 2 * A_BYTES + B_BYTES);
+      const int q = g.parts > 1 ? kt / g.kt_per : 0;
+      const uint32_t first = g.parts > 1 ? uint32_t(kt == q * g.kt_per) : uint32_t(kt == 0);
+      const uint32_t acc_t = tmem + uint32_t(q) * NCOL;
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
         const uint64_t o = uint64_t(kk * 2);   // 32 bytes >> 4
-        const uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
+        const uint32_t acc = (!first || kk > 0) ? 1u : 0u;
         if (g.bf16) {
-          mma_f16(tmem, da + o, db + o, idesc, acc);
+          mma_f16(acc_t, da + o, db + o, idesc, acc);
           if (g.split) {
-            mma_f16(tmem, da + o, dbl + o, idesc, 1u);
-            mma_f16(tmem, dal + o, db + o, idesc, 1u);
+            mma_f16(acc_t, da + o, dbl + o, idesc, 1u);
+            mma_f16(acc_t, dal + o, db + o, idesc, 1u);
           }
         } else {
-          mma_tf32(tmem, da + o, db + o, idesc, acc);
+          mma_tf32(acc_t, da + o, db + o, idesc, acc);
           if (g.split) {
-            mma_tf32(tmem, da + o, dbl + o, idesc, 1u);
-            mma_tf32(tmem, dal + o, db + o, idesc, 1u);
+            mma_tf32(acc_t, da + o, dbl + o, idesc, 1u);
+            mma_tf32(acc_t, dal + o, db + o, idesc, 1u);
           }
         }
       }
@@ -350,25 +433,38 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const __grid_constant__ 
     for (int c0 = 0; c0 < BN; c0 += 16) {
       uint32_t r[16];
       tmem_ld16(tmem + (uint32_t(warp * 32) << 16) + uint32_t(c0), r);
-      if (!g.cols_fast) {
+      for (int q = 1; q < g.parts; ++q) {
+        uint32_t u[16];
+        tmem_ld16(tmem + (uint32_t(warp * 32) << 16) + uint32_t(q) * NCOL + uint32_t(c0), u);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(u[j]));
+      }
+      float v[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]) * alpha;
+      if (EX) finish_run(g, m0 + row, n0 + c0, bias_s + c0, v);
+      if (g.cols_fast == 2) {
+        // runs of 16 columns: every lane writes its row's
+        if (om >= 0 && offn[c0] >= 0) put_run(g, pb, om + offn[c0], v);
+      } else if (g.cols_fast == 0) {
         // one row per lane: coalesced when consecutive rows are adjacent in C
         if (om < 0) continue;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           const long long on = offn[c0 + j];
-          if (on >= 0) put(om + on, __uint_as_float(r[j]) * alpha);
+          if (on >= 0) put(om + on, v[j]);
         }
       } else {
         // through shared memory: 16 lanes per row along the columns
 #pragma unroll
-        for (int j = 0; j < 16; ++j) stage_out[warp][lane][j] = __uint_as_float(r[j]);
+        for (int j = 0; j < 16; ++j) stage_out[warp][lane][j] = v[j];
         __syncwarp();
         const int j = lane & 15;
         const long long on = offn[c0 + j];
 #pragma unroll 4
         for (int i = lane >> 4; i < 32; i += 2) {
           const long long omi = offm[warp * 32 + i];
-          if (omi >= 0 && on >= 0) put(omi + on, stage_out[warp][i][j] * alpha);
+          if (omi >= 0 && on >= 0) put(omi + on, stage_out[warp][i][j]);
         }
         __syncwarp();
       }
@@ -377,7 +473,6 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const __grid_constant__ 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
-    const uint32_t ncols = BN < 32 ? 32 : BN;
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
   }
 }
@@ -396,7 +491,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 constexpr int TCP_THREADS = 320;
 constexpr int TCP_EPI = 8;   // epilogue warps
 
-template <int BN>
+template <int BN, bool EX>
 __global__ void __launch_bounds__(TCP_THREADS) k_gemm_tc_persist(const __grid_constant__ CUtensorMap ta,
                                                                  const __grid_constant__ CUtensorMap tb,
                                                                  const __grid_constant__ CUtensorMap tal,
@@ -411,6 +506,7 @@ __global__ void __launch_bounds__(TCP_THREADS) k_gemm_tc_persist(const __grid_co
   __shared__ __align__(8) uint64_t full[TC_STAGES], empty[TC_STAGES], tfull[2], tempty[2], drain;
   __shared__ uint32_t tmem_base;
   __shared__ long long offm[TC_BM], offn[BN];
+  __shared__ float bias_s[EX ? BN : 1];
   __shared__ float stage_out[TCP_EPI][32][17];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -543,6 +639,7 @@ __global__ void __launch_bounds__(TCP_THREADS) k_gemm_tc_persist(const __grid_co
         long long o = -1;
         if (n < g.N) decomp(g.gn, n, o);
         offn[c] = o;
+        if (EX) bias_s[c] = g.bias && n < g.N ? g.bias[n] : 0.f;
       }
       asm volatile("bar.sync 1, 256;" ::: "memory");
       if (dead) continue;
@@ -558,23 +655,29 @@ __global__ void __launch_bounds__(TCP_THREADS) k_gemm_tc_persist(const __grid_co
       for (int c0 = cbeg; c0 < cend; c0 += 16) {
         uint32_t r[16];
         tmem_ld16(acc_t + uint32_t(c0), r);
-        if (!g.cols_fast) {
+        float v[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]) * alpha;
+        if (EX) finish_run(g, m0 + row, n0 + c0, bias_s + c0, v);
+        if (g.cols_fast == 2) {
+          if (om >= 0 && offn[c0] >= 0) put_run(g, pb, om + offn[c0], v);
+        } else if (g.cols_fast == 0) {
           if (om < 0) continue;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const long long on = offn[c0 + j];
-            if (on >= 0) put_out(g, pb, om + on, __uint_as_float(r[j]) * alpha);
+            if (on >= 0) put_out(g, pb, om + on, v[j]);
           }
         } else {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) stage_out[warp][lane][j] = __uint_as_float(r[j]);
+          for (int j = 0; j < 16; ++j) stage_out[warp][lane][j] = v[j];
           __syncwarp();
           const int j = lane & 15;
           const long long on = offn[c0 + j];
 #pragma unroll 4
           for (int q = lane >> 4; q < 32; q += 2) {
             const long long omi = offm[quarter * 32 + q];
-            if (omi >= 0 && on >= 0) put_out(g, pb, omi + on, stage_out[warp][q][j] * alpha);
+            if (omi >= 0 && on >= 0) put_out(g, pb, omi + on, stage_out[warp][q][j]);
           }
           __syncwarp();
         }
@@ -617,7 +720,7 @@ __global__ void __launch_bounds__(256) k_tc_splitk_reduce(const __grid_constant_
     long long om, on;
     decomp(g.gm, m, om);
     decomp(g.gn, n, on);
-    put_out(g, pb, om + on, v);
+    put_out(g, pb, om + on, finish_value(g, m, n, g.bias ? g.bias[n] : 0.f, v));
   }
 }
 
@@ -660,6 +763,10 @@ __device__ __forceinline__ void split_store(float v, const PackArgs& p, long lon
     if (p.lo) static_cast<float*>(p.lo)[d] = round_tf32(v - h);
   }
 }
+__device__ __forceinline__ void split_store(__nv_bfloat16 v, const PackArgs& p, long long d) {
+  split_store(__bfloat162float(v), p, d);
+}
+
 // The same values for FP64 sources, rounded on the bits: v is an integer
 // mv = (1, mantissa) times 2^(ex - 52); h takes its leading bits, rounded to
 // nearest even (for TF32 through FP32 first, as the conversions do), and the
@@ -775,6 +882,22 @@ __global__ void __launch_bounds__(256) k_pack(const __grid_constant__ PackArgs p
     const int r = ty + TY * q, k = tx;
     if (ro[r] < 0 || ko[k] < 0) continue;
     split_store(tile[k][r], p, (pb * p.pad + r0 + r) * p.ld + k0 + k);
+  }
+}
+
+// An FP32 matrix whose rows are already contiguous along K (K a multiple of 4),
+// rounded to BF16: a copy, four values a thread, bound by HBM (50000 x 544: the
+// tiled transpose moved it at 2.7 TB/s).
+__global__ void __launch_bounds__(256) k_pack_rows(const float4* __restrict__ src, long long quads, FastDiv per_row,
+                                                   long long ld4, uint2* __restrict__ dst) {
+  for (long long t = blockIdx.x * 256LL + threadIdx.x; t < quads; t += gridDim.x * 256LL) {
+    const unsigned r = fast_div(unsigned(t), per_row), k = unsigned(t) - r * per_row.d;
+    const float4 v = src[t];
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+    uint2 o;
+    o.x = *reinterpret_cast<const unsigned*>(&a);
+    o.y = *reinterpret_cast<const unsigned*>(&b);
+    dst[r * ld4 + k] = o;
   }
 }
 
@@ -918,10 +1041,22 @@ Operand pack(Ctx& cx, const TP& src, int np, long long pad, int src_f64, const s
   const long long tiles = tiles_of(small ? 32 : 64);
   PEPS_REQUIRE(tiles < (1LL << 31), "operand too large to pack");
   const double moved = double(np) * double(o.rows) * double(o.K) *
-                       ((src_f64 ? 8.0 : 4.0) + (split ? 2.0 : 1.0) * (bf16 ? 2.0 : 4.0));
+                       ((src_f64 == 2 ? 2.0 : src_f64 ? 8.0 : 4.0) + (split ? 2.0 : 1.0) * (bf16 ? 2.0 : 4.0));
   Launch L(K_PACK, cx.st, 0, moved);
   const dim3 grid(unsigned(tiles), np);
-  if (src_f64) {
+  if (src_f64 == 0 && bf16 && !split && np == 1 && p.gr.n <= 1 && p.gk.n <= 1 && o.K % 4 == 0 &&
+      (p.gk.n == 0 || p.gk.s[0] == 1) && (p.gr.n == 0 || p.gr.s[0] == o.K) &&
+      (reinterpret_cast<uintptr_t>(src.v(0)) & 15) == 0) {
+    const long long quads = o.rows * (o.K / 4);
+    PEPS_REQUIRE(quads < (1LL << 31), "operand too large to pack");
+    k_pack_rows<<<unsigned(std::min<long long>((quads + 255) / 256, 8 * 152)), 256, 0, cx.st>>>(
+        static_cast<const float4*>(src.v(0)), quads, fast_divisor(o.K / 4), o.ld / 4, static_cast<uint2*>(o.hi));
+  } else if (src_f64 == 2) {
+    if (small)
+      k_pack<__nv_bfloat16, 32><<<grid, 256, 0, cx.st>>>(p);
+    else
+      k_pack<__nv_bfloat16, 64><<<grid, 256, 0, cx.st>>>(p);
+  } else if (src_f64) {
     if (small)
       k_pack<double, 32><<<grid, 256, 0, cx.st>>>(p);
     else
@@ -944,7 +1079,7 @@ size_t pack_words(long long rows, long long K, int bf16, int split) {
   return split ? 2 * words : words;
 }
 
-template <int BN>
+template <int BN, bool EX>
 void launch_tc(Ctx& cx, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tal,
                const CUtensorMap& tbl, TcArgs g, long long tiles) {
   const int a_bytes = TC_BM * TC_ROWB, b_bytes = BN * TC_ROWB;
@@ -956,8 +1091,8 @@ void launch_tc(Ctx& cx, const CUtensorMap& ta, const CUtensorMap& tb, const CUte
   static int nsm = 0;
   static bool persist = true;   // PEPS_TC_PERSIST=0 keeps every GEMM on the one-tile kernel
   std::call_once(once, [] {
-    PEPS_CUDA(cudaFuncSetAttribute(k_gemm_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    PEPS_CUDA(cudaFuncSetAttribute(k_gemm_tc_persist<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    PEPS_CUDA(cudaFuncSetAttribute(k_gemm_tc<BN, EX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    PEPS_CUDA(cudaFuncSetAttribute(k_gemm_tc_persist<BN, EX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     int dev = 0;
     PEPS_CUDA(cudaGetDevice(&dev));
     PEPS_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -965,13 +1100,13 @@ void launch_tc(Ctx& cx, const CUtensorMap& ta, const CUtensorMap& tb, const CUte
   });
   if (!persist || g.splitk > 1 || tiles <= nsm) {
     // split-K partials, or no more tiles than SMs: one tile per CTA
-    k_gemm_tc<BN><<<dim3(unsigned(tiles), unsigned(std::max(1, g.splitk))), TC_THREADS, smem, cx.st>>>(ta, tb, tal,
+    k_gemm_tc<BN, EX><<<dim3(unsigned(tiles), unsigned(std::max(1, g.splitk))), TC_THREADS, smem, cx.st>>>(ta, tb, tal,
                                                                                                         tbl, g);
   } else {
     // the ring holds at least two stages so the next tile's operands stream in
     g.stages = std::max(1, std::min(TC_STAGES, (budget - 1024) / stage));
     const size_t psmem = size_t(stage) * g.stages + 1024;
-    k_gemm_tc_persist<BN><<<unsigned(nsm), TCP_THREADS, psmem, cx.st>>>(ta, tb, tal, tbl, g);
+    k_gemm_tc_persist<BN, EX><<<unsigned(nsm), TCP_THREADS, psmem, cx.st>>>(ta, tb, tal, tbl, g);
   }
   PEPS_CHECK_LAUNCH();
 }
@@ -1035,7 +1170,7 @@ void ein_tc(Ctx& cx, const char* spec, const TP& A, int a_f64, const Dims& ad, c
             const Dims& bd, const TP& C, int c_f64, int prec, double alpha, const TP& Clo, PackCache* bcache,
             const TcChain* chain) {
   PEPS_REQUIRE(tc_available(), "tensor-core path needs an sm_103 device");
-  const bool to_next = chain && chain->next;
+  const bool to_next = chain && chain->next;   // a chain without `next` may still bring a bias, relu or mask
   const TcOperand* a_pre = chain ? chain->a_pre : nullptr;
   int np = to_next ? problems({&A, &B}) : problems({&A, &B, &C, &Clo});
   if (a_pre) {
@@ -1129,14 +1264,25 @@ void ein_tc(Ctx& cx, const char* spec, const TP& A, int a_f64, const Dims& ad, c
   PEPS_REQUIRE(tiles < (1LL << 31), "too many tiles");
   g.ktiles = int((K + (TC_ROWB / (bf16 ? 2 : 4)) - 1) / (TC_ROWB / (bf16 ? 2 : 4)));
   // Split K when the output tiles would leave most SMs idle: each split runs
-  // at least two k tiles; partials are reduced in a fixed order.
+  // at least two k tiles; partials are reduced in a fixed order.  In plain BF16,
+  // up to 16 k tiles and four splits, one CTA takes them all, each into an
+  // accumulator of its own in TMEM, added in the same order (the same results
+  // bit for bit): it multiplies 16 tiles in 3 us, the kernel that adds partials
+  // takes 5.  Not in the split precisions, whose three products per tile and
+  // twice the operands take longer than that (a TF32x3 plan: 104 ms, 115 so).
   g.splitk = 1;
   g.kt_per = g.ktiles;
+  const bool extras = chain && (chain->bias || chain->relu || chain->mask);
+  g.parts = 1;
   if (tiles < 152 && g.ktiles >= 4) {
     const long long want = std::min<long long>((2 * 152 + tiles - 1) / tiles, g.ktiles / 2);
     if (want > 1) {
       g.kt_per = int((g.ktiles + want - 1) / want);
       g.splitk = int((g.ktiles + g.kt_per - 1) / g.kt_per);
+    }
+    if (bf16 && !split && g.splitk > 1 && g.splitk <= 4 && g.splitk * std::max(BN, 32) <= 512 && g.ktiles <= 16) {
+      g.parts = g.splitk;
+      g.splitk = 1;
     }
   }
   const size_t wp = g.splitk > 1 ? (size_t(g.splitk) * np * M * N + 1) / 2 + 64 : 0;
@@ -1233,12 +1379,30 @@ void ein_tc(Ctx& cx, const char* spec, const TP& A, int a_f64, const Dims& ad, c
     };
     const long long sc_cols = sectors(true), sc_rows = sectors(false);
     g.cols_fast = sc_cols != sc_rows ? (sc_cols < sc_rows ? 1 : 0) : (inner(g.gn) < inner(g.gm) ? 1 : 0);
+    // Every 16 aligned columns one aligned run of the output: each lane stores
+    // its row's run in 16-byte pieces (whole sectors, no staging).
+    auto aligned = [&](const TP& t) {
+      for (int b = 0; b < t.n; ++b)
+        if (reinterpret_cast<uintptr_t>(t.p[b]) & 15) return false;
+      return true;
+    };
+    bool runs = g.gn.n > 0 && g.gn.s[g.gn.n - 1] == 1 && g.gn.dim[g.gn.n - 1].d % 16 == 0 && aligned(g.C) &&
+                aligned(g.Clo);
+    for (int i = 0; i + 1 < g.gn.n; ++i) runs = runs && g.gn.s[i] % 8 == 0;
+    for (int i = 0; i < g.gm.n; ++i) runs = runs && g.gm.s[i] % 8 == 0;
+    if (runs) g.cols_fast = 2;
   }
   g.nprob = np;
   g.pad_m = pad_m;
   g.pad_n = pad_n;
   g.alpha = alpha;
   g.flag = cx.flag;
+  if (extras) {
+    PEPS_REQUIRE(np == 1, "internal: bias or mask with several problems");
+    g.bias = chain->bias;
+    g.mask = static_cast<const __nv_bfloat16*>(chain->mask);
+    g.relu = chain->relu ? 1 : 0;
+  }
   const double flops = 2.0 * double(M) * double(N) * double(K) * np;
   // algorithmic bytes: both packed operands read once, the output written once
   // (as the next contraction's packed operand, FP64, or FP32 with its residual)
@@ -1246,11 +1410,18 @@ void ein_tc(Ctx& cx, const char* spec, const TP& A, int a_f64, const Dims& ad, c
   const double out_b = to_next ? in_b : (g.out_f64 ? 8.0 : (g.out_lo ? 8.0 : 4.0));
   const double bytes = double(np) * (double(M) * K * in_b + double(N) * K * in_b + double(M) * N * out_b);
   Launch L(K_GEMM_TC, cx.st, flops, bytes);
+  auto run = [&](auto bn) {
+    constexpr int N_ = decltype(bn)::value;
+    if (extras)
+      launch_tc<N_, true>(cx, ta, tb, tal, tbl, g, tiles);
+    else
+      launch_tc<N_, false>(cx, ta, tb, tal, tbl, g, tiles);
+  };
   switch (BN) {
-    case 16: launch_tc<16>(cx, ta, tb, tal, tbl, g, tiles); break;
-    case 32: launch_tc<32>(cx, ta, tb, tal, tbl, g, tiles); break;
-    case 64: launch_tc<64>(cx, ta, tb, tal, tbl, g, tiles); break;
-    default: launch_tc<128>(cx, ta, tb, tal, tbl, g, tiles); break;
+    case 16: run(std::integral_constant<int, 16>()); break;
+    case 32: run(std::integral_constant<int, 32>()); break;
+    case 64: run(std::integral_constant<int, 64>()); break;
+    default: run(std::integral_constant<int, 128>()); break;
   }
   if (g.splitk > 1) {
     const unsigned blocks = unsigned(std::max<long long>(1, std::min<long long>((M * N + 255) / 256, 4096)));

@@ -133,3 +133,55 @@ def test_recorded_plan_with_learned_closure(env):
     e = plan.run()
     for kind, op in (("site", O.SZ), ("hbond", O.SDOTS), ("vbond", O.SDOTS)):
         assert np.max(np.abs(plain.expect(kind, op) - e.expect(kind, op))) < 1e-12
+
+
+def _network_with_bf16_operands(torch, w, X, Y, F, W, D):
+    """Loss, gradient and sigma in FP64 with every GEMM operand rounded to BF16."""
+    def r(t):
+        return t.float().bfloat16().double()
+    o, n = D * D, X.shape[0]
+    W1, b1, W2, b2, W3, b3 = torch.split(w.double(), [W * F, W, W * W, W, o * W, o])
+    W1, W2, W3, x = W1.reshape(W, F), W2.reshape(W, W), W3.reshape(o, W), X.double()
+    H1 = torch.relu(r(x) @ r(W1).T + b1)
+    H2 = torch.relu(r(H1) @ r(W2).T + b2)
+    Yo = (r(H2) @ r(W3).T + b3).float().double()
+    M = x[:, F - o:].reshape(-1, D, D) + Yo.reshape(-1, D, D)
+    S = M @ M.mT
+    nr = S.square().sum((1, 2), keepdim=True).sqrt()
+    sig = S / nr
+    df = sig - Y.double().reshape(-1, D, D)
+    G = 2 * df / n
+    dS = (G - sig * (G * sig).sum((1, 2), keepdim=True)) / nr
+    dY = ((dS + dS.mT) @ M).reshape(n, o).float().double()
+    dH2 = (r(dY) @ r(W3)) * (H2 > 0)
+    dH1 = (r(dH2) @ r(W2)) * (H1 > 0)
+    grad = torch.cat([(r(dH1).T @ r(x)).reshape(-1), dH1.sum(0), (r(dH2).T @ r(H1)).reshape(-1), dH2.sum(0),
+                      (r(dY).T @ r(H2)).reshape(-1), dY.sum(0)])
+    return float(df.square().sum() / n), grad, sig.reshape(n, o)
+
+
+@pytest.mark.parametrize("D,n", [(2, 1), (2, 127), (3, 129), (4, 300), (5, 200), (6, 40), (8, 33)])
+def test_gradient_and_inference_at_batch_edges(env, D, n):
+    """One example, partial tiles, and widths whose layers split K inside a CTA
+    (D = 4) and over several (D >= 5), against the same network with its GEMM
+    operands rounded to BF16.  What is left is FP32 accumulation, ~1e-5 of a
+    row, which moves an operand to its other BF16 neighbour (2^-8) with
+    probability ~3e-3: 2e-4 of a layer's norm, 1e-3 after six GEMMs; a small
+    sigma - label multiplies that by up to ten."""
+    torch, peps = env
+    W, F = 256, 2 * D ** 4 + 2 * D * D
+    g = torch.Generator().manual_seed(7 * D + n)
+    low = torch.tril(0.2 * torch.randn(n, D, D, generator=g, dtype=torch.float64), -1) + torch.eye(D, dtype=torch.float64)
+    low = low / (low @ low.mT).square().sum((1, 2), keepdim=True).sqrt().sqrt()
+    site = torch.randn(n, 2 * D ** 4, generator=g, dtype=torch.float64)
+    X = torch.cat([site / site.norm(dim=1, keepdim=True), (low @ low.mT).reshape(n, -1), low.reshape(n, -1)], 1).float()
+    Y = torch.eye(D).reshape(1, -1).repeat(n, 1) / D ** 0.5
+    w = peps.mlp_init(2, D, seed=D)
+    k = W * F + W + W * W + W
+    w[k:] = 0.05 * torch.randn(D * D * W + D * D, generator=g).cuda()
+    w[W * F:W * F + W] = 0.1 * torch.randn(W, generator=g).cuda()
+    loss, grad = peps.mlp_loss_grad(w, X.cuda(), Y.cuda(), 2, D)
+    want_loss, want, sig = _network_with_bf16_operands(torch, w.cpu(), X, Y, F, W, D)
+    assert abs(loss - want_loss) < 1e-2 * abs(want_loss)
+    assert _rel(grad.cpu().double().numpy(), want.numpy()) < 1e-2
+    assert np.max(np.abs(peps.mlp_predict(w, X.cuda(), 2, D).cpu().double().numpy() - sig.numpy())) < 1e-3
