@@ -282,6 +282,7 @@ struct Call {
     cx.cu0_cap = fault.mode == FAULT_CONVERGE ? 1 : cap_cu0_half_sweeps();
     if (const char* e = std::getenv("PEPS_QR_CMAX")) cx.qr_cmax = std::atoi(e);
     if (tune.qr_cmax > 0) cx.qr_cmax = tune.qr_cmax;
+    cx.qr_whole = true;   // the lanes' own contexts leave it off
     cx.flag = static_cast<int*>(persist ? persist->alloc(sizeof(int)) : ws.alloc(sizeof(int)));
     PEPS_CUDA(cudaMemsetAsync(cx.flag, 0, sizeof(int), st));
     cx.tmp = ws.dalloc(8);

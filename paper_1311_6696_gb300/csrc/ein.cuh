@@ -24,6 +24,8 @@ struct Ctx {
   Arena* persist = nullptr;
   // Largest thread-block cluster a QR may use (0: no limit beyond 16).
   int qr_cmax = 0;
+  // A QR may take every SM: no other stream of this call has work beside it.
+  bool qr_whole = false;
   // Iteration caps of this call (Jacobi SVD sweeps, CU_0 half-sweeps).
   int svd_cap = 60;
   int cu0_cap = 200;

@@ -62,7 +62,15 @@ struct QrArgs {
   double* Qw;   // k_qr_house: m*k work per problem, column-major (+ p * qst)
   double* tau;  // k_qr_house: k per problem (+ p * tst)
   long long wst, qst, tst;
+  // k_qr_cluster over G clusters per problem (absent otherwise):
+  int G;
+  double* gsum;      // [problem][2][G][n] the clusters' partial sums
+  double* grow;      // [problem][2][n] row j of the matrix
+  unsigned* gcount;  // [problem][QRG_LINE] arrivals, zero at launch
+  int* flag;
 };
+constexpr int QRG_LINE = 32;   // counters 128 bytes apart
+constexpr int QRG_MAX = 20;    // clusters per problem: five sums per thread
 
 // Grid = problems, one CTA each, everything in global memory: for matrices with
 // more columns than k_qr_cluster's shared memory holds sums for.
@@ -202,6 +210,18 @@ __device__ __forceinline__ double remote_sum(cg::cluster_group& cl, double* slot
 // 3847 -> 2853; 16 of 36x36 270 -> 123 (those ran in global memory, one CTA
 // each).  Orthogonality stays at 1e-15 to 7e-15; |A - QR| is 1 to 3 eps of a
 // column's norm.
+//
+// GRID: the rows of one matrix over G clusters.  One cluster has 16 SMs, and
+// of clusters of 16 only seven run at once, so that one matrix, or its leaves,
+// left more than half of the chip idle.  After the cluster's barrier each CTA
+// sums its share of the columns over the cluster and writes it, one value per
+// column and cluster, to global memory; the clusters' arrivals are counted
+// there, and every CTA then adds the G values itself.  That wait costs a column
+// about 5000 clocks more (an L2 round trip to publish, one or two to see the
+// count, one to read), so it pays where the rows of 16 CTAs cost more than that.
+// Measured (us, one cluster or leaves -> clusters): 2304x64 619 -> 423,
+// 1024x128 1127 -> 776, 4096x128 2069 -> 1010, 8192x128 2801 -> 1362,
+// 1620x180 2863 -> 1602, 8192x64 861 -> 625, three of 4096x128 2781 -> 1547.
 // ---------------------------------------------------------------------------
 constexpr int QRC_MAXT = 512;
 
@@ -266,23 +286,47 @@ __device__ __forceinline__ double qr_update_dot(double* wc, const double* xj, co
   return acc;
 }
 
+__device__ __forceinline__ void arrive_gpu(unsigned* p) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+__device__ __forceinline__ unsigned load_acquire_gpu(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+// Bounded wait (about 2 s of SM clock) for `target` arrivals: false, with the
+// status word set, when it runs out.
+__device__ __forceinline__ bool wait_arrivals(const unsigned* p, unsigned target, int* flag) {
+  const long long start = clock64();
+  while (int(load_acquire_gpu(p) - target) < 0) {
+    if (clock64() - start > 4000000000LL) {
+      atomicOr(flag, FLAG_TIMEOUT);
+      return false;
+    }
+  }
+  return true;
+}
+
 // lanes_log2: threads that share a column of the pass, 4 to 32: 128 threads
 // are enough to keep the FP64 pipe busy, and each doubling adds an addition to
 // every sum.
+template <bool GRID>
 __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_smem, int tri_smem, int ld,
                                                          int lanes_log2) {
   extern __shared__ double qsm[];
   cg::cluster_group cluster = cg::this_cluster();
   const int C = int(cluster.num_blocks());
   const int rank = int(cluster.block_rank());
-  const int pb = blockIdx.x / C;               // one cluster per problem
+  const int G = GRID ? q.G : 1;                // clusters per problem
+  const int pb = blockIdx.x / (C * G);
+  const int gid = GRID ? blockIdx.x / C - pb * G : 0;
   const double* A = q.A.d(pb);
   double* const Qo = q.Q.d(pb);
   double* const Ro = q.R.n ? q.R.d(pb) : nullptr;
   const int m = q.m, n = q.n, k = min(m, n);
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-  const int chunk = (m + C - 1) / C;
-  const int r0 = min(m, rank * chunk), r1 = min(m, r0 + chunk), rows = r1 - r0;
+  const int chunk = (m + C * G - 1) / (C * G);
+  const int r0 = min(m, (gid * C + rank) * chunk), r1 = min(m, r0 + chunk), rows = r1 - r0;
   const int mcols = (k + C - 1) / C;        // columns of M solved here: rank, rank + C, ...
   double* part = qsm;                       // [2][n] my partial sums (read by every CTA)
   double* rowv = part + 2 * n;              // [2][n] row j of the matrix (in the row's owner)
@@ -296,7 +340,10 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
   double* mc = vs + k + 4;                  // [mcols][k] my columns of X_1^T, then of M (read by every CTA)
   double* tri = mc + mcols * k;             // packed columns: X^T X above the diagonal, then M
   double* W = tri + (tri_smem ? qr_tri(k) : 0);   // [n][ld], row i at i - r0
-  {
+  double* const gsum = GRID ? q.gsum + (long long)pb * 2 * G * n : nullptr;
+  double* const grow = GRID ? q.grow + (long long)pb * 2 * n : nullptr;
+  bool live = true;                         // the polling thread: no wait has run out
+  if (!GRID) {
     double* g = q.W + pb * q.wst + rank * (q.wst / C);
     if (!tri_smem) {
       tri = g;
@@ -345,38 +392,74 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
       for (int o = L >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
       if (c < n && l == 0) {
         part[b * n + c] = acc;
-        if (own) rowv[b * n + c] = wc[jn];
+        if (own) {
+          if (GRID)
+            __stcg(grow + b * n + c, wc[jn]);
+          else
+            rowv[b * n + c] = wc[jn];
+        }
       }
     }
   };
+  // Sum over the cluster of one partial sum, by four neighbouring lanes (l: which of them).
+  auto cluster_sum = [&](double* slot, int l) {
+    const double v0 = l < C ? *cluster.map_shared_rank(slot, l) : 0.0;
+    const double v1 = l + 4 < C ? *cluster.map_shared_rank(slot, l + 4) : 0.0;
+    const double v2 = l + 8 < C ? *cluster.map_shared_rank(slot, l + 8) : 0.0;
+    const double v3 = l + 12 < C ? *cluster.map_shared_rank(slot, l + 12) : 0.0;
+    double s = v0;
+    if (C > 4) s += v1;
+    if (C > 8) s = (s + v2) + v3;
+    if (C > 2) s += __shfl_xor_sync(0xffffffffu, s, 2);
+    return s + __shfl_xor_sync(0xffffffffu, s, 1);
+  };
+  const int slice = (n + C - 1) / C;                  // GRID: columns whose sums over the cluster this CTA takes
+  const unsigned arrivals = unsigned(G * C) * unsigned((4 * slice + 31) / 32);   // warps that publish, per step
   pass(-1, 0, 0);
   for (int j = 0; j < k; ++j) {
     const int b = j & 1, owner = j / chunk;
     cta_or_cluster_sync();                            // column j: inner products and row j visible
+    if (GRID) {
+      for (int t0 = tid - lane; t0 < 4 * slice; t0 += nt) {
+        const int ci = (t0 + lane) >> 2, l = lane & 3, c = rank * slice + ci;
+        const double s = cluster_sum(part + b * n + min(c, n - 1), l);
+        if (l == 0 && ci < slice && c < n) __stcg(gsum + (b * G + gid) * n + c, s);
+        __syncwarp();
+        if (lane == 0) arrive_gpu(q.gcount + pb * QRG_LINE);
+      }
+      // both buffers are free again two steps on: an arrival follows its warp's reads
+      if (tid == nt - 32 && live) live = wait_arrivals(q.gcount + pb * QRG_LINE, unsigned(j + 1) * arrivals, q.flag);
+      __syncthreads();
+    }
     // row j, local copy: the threads that do not sum start at the far end
     for (int c = nt - 1 - tid; c < n; c += nt)
-      rowl[c] = C > 1 ? *cluster.map_shared_rank(rowv + b * n + c, owner) : rowv[b * n + c];
-    // sums over the CTAs, four threads per column, column j first
+      rowl[c] = GRID    ? __ldcg(grow + b * n + c)
+                : C > 1 ? *cluster.map_shared_rank(rowv + b * n + c, owner)
+                        : rowv[b * n + c];
+    // sums over the CTAs (or clusters), four threads per column, column j first
     for (int t0 = tid - lane; t0 < 4 * n; t0 += nt) {
       const int ci = (t0 + lane) >> 2, l = lane & 3;
       int c = min(ci, n - 1) + j;
       if (c >= n) c -= n;
       double* slot = part + b * n + c;
       double alpha = 0.0, s;
-      if (C == 1) {
+      if (GRID) {
+        double v[QRG_MAX / 4];
+#pragma unroll
+        for (int i = 0; i < QRG_MAX / 4; ++i) v[i] = 4 * i + l < G ? __ldcg(gsum + (b * G + 4 * i + l) * n + c) : 0.0;
+        if (ci == 0) alpha = __ldcg(grow + b * n + j);
+        s = v[0];
+#pragma unroll
+        for (int i = 1; i < QRG_MAX / 4; ++i)
+          if (4 * i < G) s += v[i];
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+      } else if (C == 1) {
         s = *slot;
         if (ci == 0) alpha = rowv[b * n + j];
       } else {
-        const double v0 = l < C ? *cluster.map_shared_rank(slot, l) : 0.0;
-        const double v1 = l + 4 < C ? *cluster.map_shared_rank(slot, l + 4) : 0.0;
-        const double v2 = l + 8 < C ? *cluster.map_shared_rank(slot, l + 8) : 0.0;
-        const double v3 = l + 12 < C ? *cluster.map_shared_rank(slot, l + 12) : 0.0;
         if (ci == 0) alpha = *cluster.map_shared_rank(rowv + b * n + j, owner);
-        s = v0;
-        if (C > 4) s += v1;
-        if (C > 8) s = (s + v2) + v3;
-        if (C > 2) s += __shfl_xor_sync(0xffffffffu, s, 2);
-        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s = cluster_sum(slot, l);
       }
       if (ci >= n || l != 0) continue;
       if (ci > 0) {
@@ -849,6 +932,24 @@ int qr_lanes_log2(int n) { return n > 16 ? 2 : n > 8 ? 3 : n > 4 ? 4 : 5; }
 
 size_t qr_tri_bytes(int m, int n) { return sizeof(double) * size_t(qr_tri(std::min(m, n))); }
 
+// A launch on clusters of c CTAs.
+struct ClusterLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  ClusterLaunch(int ctas, int threads, size_t smem, int c, cudaStream_t st) {
+    cfg.gridDim = dim3(ctas, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = c;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+};
+
 // Estimated clocks of np factorisations on clusters of c CTAs, fitted to
 // measured times of shapes from 16x16 to 2304x64 on 1 to 16 CTAs (within 20%):
 // a column costs its barriers, sums and scalars, its share of the back
@@ -862,7 +963,7 @@ double qr_clocks(int m, int n, int c, int np) {
   const double warps = qr_threads(n) / 32;
   const size_t rows_b = qr_smem(m, n, c), all_b = rows_b + qr_tri_bytes(m, n);
   const bool tri = all_b <= kQrSmemMax;
-  const int at_once = active_clusters(k_qr_cluster, qr_threads(n), tri ? all_b : rows_b, c);
+  const int at_once = active_clusters(k_qr_cluster<false>, qr_threads(n), tri ? all_b : rows_b, c);
   if (at_once == 0) return 1e300;
   const double step = (c == 1 ? 3800.0 : 5600.0) + 180.0 * std::ceil(std::ceil(k / c) / warps);
   const double fp = 24.0 * rows * 2.0 * n / 32.0 * (n < 64 ? 1.3 : 1.0);
@@ -938,7 +1039,7 @@ QrPlan qr_plan(int m, int n, int np, int qr_cmax) {
   };
   while (p.C > 0) {
     settle();
-    if (active_clusters(k_qr_cluster, qr_threads(n), p.bytes, p.C) > 0) break;
+    if (active_clusters(k_qr_cluster<false>, qr_threads(n), p.bytes, p.C) > 0) break;
     p.C /= 2;   // clusters of this size cannot be launched here
     p.w_smem = p.C > 0 && qr_smem(m, n, p.C) <= kQrSmemMax;
     if (p.C > 0 && qr_head_bytes(m, n, p.C) > kQrSmemMax) p.C = 0;
@@ -968,21 +1069,65 @@ int tsqr_leaves(int m, int n, int np, double* clocks) {
   return best;
 }
 
-// Leaves of m x n (0: none), kept per shape.
-int tsqr_plan(int m, int n, int np) {
+// How a matrix with m >= 1024 rows is factored: over G clusters of C CTAs at
+// once (G > 0), in L leaves (L > 0), or like any other.
+struct TallPlan {
+  int L = 0;
+  int C = 0, G = 0;
+  size_t bytes = 0;
+};
+
+// k_qr_cluster<true> on the shape with the least estimated time (G = 0: none):
+// qr_clocks' terms with the wait for the other clusters in every column (10500
+// clocks where one cluster has 5600; 1024x128 to 8192x128 come out within 15%,
+// 180 columns a quarter low).  Rows and triangle in shared memory, one CTA per
+// SM at most, and no more clusters than run at once.
+TallPlan qr_grid(int m, int n, int np, double* clocks) {
+  TallPlan p;
+  *clocks = 1e300;
+  int dev = 0, sms = 0;
+  PEPS_CUDA(cudaGetDevice(&dev));
+  PEPS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const double warps = qr_threads(n) / 32;
+  for (int c = 4; c <= 16; c *= 2) {
+    int g = std::min(QRG_MAX, sms / c / np);
+    for (bool fits = false; g > 1 && !fits; g -= fits ? 0 : 1) {
+      const size_t b = qr_smem(m, n, c * g) - qr_head_bytes(m, n, c * g) + qr_head_bytes(m, n, c) + qr_tri_bytes(m, n);
+      fits = b <= kQrSmemMax && active_clusters(k_qr_cluster<true>, qr_threads(n), b, c) >= g * np;
+      if (!fits) continue;
+      const double rows = std::ceil(double(m) / (c * g));
+      const double step = 10500.0 + 180.0 * std::ceil(std::ceil(double(n) / c) / warps);
+      const double t = 14000.0 + n * (step + 24.0 * rows * 2.0 * n / 32.0 * (n < 64 ? 1.3 : 1.0));
+      if (t < *clocks) {
+        *clocks = t;
+        p.C = c;
+        p.G = g;
+        p.bytes = b;
+      }
+    }
+  }
+  return p;
+}
+
+// Kept per shape.
+TallPlan tall_plan(int m, int n, int np, bool whole) {
   static std::mutex mu;
-  static std::map<std::tuple<int, int, int, int>, int> cache;
+  static std::map<std::tuple<int, int, int, int, bool>, TallPlan> cache;
   int dev = 0;
   PEPS_CUDA(cudaGetDevice(&dev));
-  const auto key = std::make_tuple(dev, m, n, np);
+  const auto key = std::make_tuple(dev, m, n, np, whole);
   std::lock_guard<std::mutex> g(mu);
   const auto it = cache.find(key);
   if (it != cache.end()) return it->second;
-  double direct, leaves;
+  double direct, leaves, grid = 1e300;
   qr_best_cluster(m, n, np, 16, &direct);
-  const int L = tsqr_leaves(m, n, np, &leaves);
+  TallPlan p, w;
+  p.L = tsqr_leaves(m, n, np, &leaves);
+  if (whole) w = qr_grid(m, n, np, &grid);
   // the estimates are no better than a tenth
-  return cache.emplace(key, L > 1 && leaves < 0.9 * direct ? L : 0).first->second;
+  if (!(p.L > 1 && leaves < 0.9 * direct)) p.L = 0;
+  if (w.G > 0 && grid < 0.9 * (p.L ? leaves : direct)) p = w;
+  return cache.emplace(key, p).first->second;
 }
 
 }  // namespace
@@ -1045,6 +1190,39 @@ void qr_tsqr(Ctx& cx, int m, int n, int L, const TP& A, long long rs, long long 
   }
 }
 
+// One QR over G clusters.  Cooperative: its clusters wait for one another and
+// have to be resident together.
+void qr_clusters(Ctx& cx, int m, int n, const TallPlan& p, const TP& A, long long rs, long long cs, const TP& Q,
+                 long long qrs, long long qcs, const TP& R, int np) {
+  QrArgs a;
+  std::memset(static_cast<void*>(&a), 0, sizeof(a));
+  a.m = m;
+  a.n = n;
+  a.A = A.all(np);
+  a.rs = rs;
+  a.cs = cs;
+  a.Q = Q.all(np);
+  a.qrs = qrs;
+  a.qcs = qcs;
+  a.R = R.all(np);
+  a.G = p.G;
+  a.flag = cx.flag;
+  const size_t count = size_t(np) * QRG_LINE / 2, sums = size_t(np) * 2 * p.G * n, rows = size_t(np) * 2 * n;
+  double* w = cx.scratch(count + sums + rows);
+  a.gcount = reinterpret_cast<unsigned*>(w);
+  a.gsum = w + count;
+  a.grow = a.gsum + sums;
+  PEPS_CUDA(cudaMemsetAsync(a.gcount, 0, count * sizeof(double), cx.st));
+  if (std::getenv("PEPS_VERBOSE")) std::fprintf(stderr, "[peps] qr %dx%d x%d: %d clusters of %d\n", m, n, np, p.G, p.C);
+  Launch L(K_QR, cx.st, qr_flops(m, n) * np, 0);
+  ClusterLaunch c(p.C * p.G * np, qr_threads(n), p.bytes, p.C, cx.st);
+  c.at[1].id = cudaLaunchAttributeCooperative;
+  c.at[1].val.cooperative = 1;
+  c.cfg.numAttrs = 2;
+  PEPS_CUDA(cudaLaunchKernelEx(&c.cfg, k_qr_cluster<true>, a, 1, 1, qr_ld(m, p.C * p.G), qr_lanes_log2(n)));
+  PEPS_CHECK_LAUNCH();
+}
+
 void qr_thin(Ctx& cx, int m, int n, const TP& A, long long rs, long long cs, const TP& Q, long long qrs,
              long long qcs, const TP& R) {
   PEPS_REQUIRE(m > 0 && n > 0, "qr of an empty matrix");
@@ -1054,9 +1232,13 @@ void qr_thin(Ctx& cx, int m, int n, const TP& A, long long rs, long long cs, con
   // do not fit in the shared memory of one cluster or the leaves are estimated
   // to be faster.
   if (m >= 1024 && m >= n && cx.qr_cmax <= 0) {
-    const int L = tsqr_plan(m, n, np);
-    if (L > 1) {
-      qr_tsqr(cx, m, n, L, A, rs, cs, Q, qrs, qcs, R, np);
+    const TallPlan p = tall_plan(m, n, np, cx.qr_whole);
+    if (p.L > 0) {
+      qr_tsqr(cx, m, n, p.L, A, rs, cs, Q, qrs, qcs, R, np);
+      return;
+    }
+    if (p.G > 0) {
+      qr_clusters(cx, m, n, p, A, rs, cs, Q, qrs, qcs, R, np);
       return;
     }
   }
@@ -1100,19 +1282,9 @@ void qr_direct(Ctx& cx, int m, int n, const TP& A, long long rs, long long cs, c
   if (C == 0) {
     k_qr_house<<<np, QR_THREADS, 0, cx.st>>>(a);
   } else {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C * np, 1, 1);
-    cfg.blockDim = dim3(qr_threads(n), 1, 1);
-    cfg.dynamicSmemBytes = pl.bytes;
-    cfg.stream = cx.st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    PEPS_CUDA(cudaLaunchKernelEx(&cfg, k_qr_cluster, a, pl.w_smem ? 1 : 0, pl.tri_smem ? 1 : 0, ld, qr_lanes_log2(n)));
+    ClusterLaunch c(C * np, qr_threads(n), pl.bytes, C, cx.st);
+    PEPS_CUDA(cudaLaunchKernelEx(&c.cfg, k_qr_cluster<false>, a, pl.w_smem ? 1 : 0, pl.tri_smem ? 1 : 0, ld,
+                                 qr_lanes_log2(n)));
   }
   PEPS_CHECK_LAUNCH();
 }

@@ -33,3 +33,16 @@ def test_norm_at_factor_edges(peps, Ly, Lx, D, chi, mode):
     A = synth.peps_gauss(Ly, Lx, 2, D, seed=40 + D)
     got, want = peps.norm(A, chi, mode=mode, seed=2), O.norm(A, chi=chi, mode=mode, seed=2)
     assert abs(got[0] - want[0]) < 1e-10 and got[1] == want[1]
+
+
+# Boundary tensors of 1024 rows and more, whose QR is split over several
+# clusters: columns that are no multiple of a warp's or a cluster's share
+# (1500x60), and more of them than four threads each cover (2240x140); just
+# below the rule, on one cluster (1008x63).  |ln N| is a few tens, and both
+# sides round in FP64 only: the 1e-10 above.
+@pytest.mark.parametrize("Ly,Lx,D,chi", [(4, 6, 5, 60), (4, 6, 4, 140), (4, 6, 4, 63)])
+def test_norm_with_tall_boundaries(peps, Ly, Lx, D, chi):
+    from paper_1311_6696_gb300 import synth
+    A = synth.peps_gauss(Ly, Lx, 2, D, seed=60 + D)
+    got, want = peps.norm(A, chi, mode="var", seed=2), O.norm(A, chi=chi, mode="var", seed=2)
+    assert abs(got[0] - want[0]) < 1e-10 and got[1] == want[1]
