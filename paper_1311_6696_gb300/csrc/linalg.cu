@@ -62,15 +62,17 @@ struct QrArgs {
   double* Qw;   // k_qr_house: m*k work per problem, column-major (+ p * qst)
   double* tau;  // k_qr_house: k per problem (+ p * tst)
   long long wst, qst, tst;
-  // k_qr_cluster over G clusters per problem (absent otherwise):
-  int G;
-  double* gsum;      // [problem][2][G][n] the clusters' partial sums
-  double* grow;      // [problem][2][n] row j of the matrix
-  unsigned* gcount;  // [problem][QRG_LINE] arrivals, zero at launch
+  // k_qr_cluster<true>, P CTAs per problem (absent otherwise), per problem:
+  int P;
+  double* gpart;     // [n][P] the CTAs' partial sums
+  double* gsum;      // [n] their sums
+  double* grow;      // [2][n] row j of the matrix
+  double* gtri;      // M, packed columns
+  unsigned* gcount;  // two counters QRG_LINE apart, zero at launch: partial sums, sums
   int* flag;
 };
-constexpr int QRG_LINE = 32;   // counters 128 bytes apart
-constexpr int QRG_MAX = 20;    // clusters per problem: five sums per thread
+constexpr int QRG_LINE = 32;    // 128 bytes
+constexpr int QRG_MAXP = 160;   // five partial sums per lane
 
 // Grid = problems, one CTA each, everything in global memory: for matrices with
 // more columns than k_qr_cluster's shared memory holds sums for.
@@ -211,17 +213,19 @@ __device__ __forceinline__ double remote_sum(cg::cluster_group& cl, double* slot
 // each).  Orthogonality stays at 1e-15 to 7e-15; |A - QR| is 1 to 3 eps of a
 // column's norm.
 //
-// GRID: the rows of one matrix over G clusters.  One cluster has 16 SMs, and
-// of clusters of 16 only seven run at once, so that one matrix, or its leaves,
-// left more than half of the chip idle.  After the cluster's barrier each CTA
-// sums its share of the columns over the cluster and writes it, one value per
-// column and cluster, to global memory; the clusters' arrivals are counted
-// there, and every CTA then adds the G values itself.  That wait costs a column
-// about 5000 clocks more (an L2 round trip to publish, one or two to see the
-// count, one to read), so it pays where the rows of 16 CTAs cost more than that.
-// Measured (us, one cluster or leaves -> clusters): 2304x64 619 -> 423,
-// 1024x128 1127 -> 776, 4096x128 2069 -> 1010, 8192x128 2801 -> 1362,
-// 1620x180 2863 -> 1602, 8192x64 861 -> 625, three of 4096x128 2781 -> 1547.
+// GRID: the rows of one matrix over every SM.  One cluster has 16 SMs, and of
+// clusters of 16 only seven run at once, so that one matrix, or its leaves,
+// left more than half of the chip idle.  The CTAs are no cluster here (a
+// cooperative launch): the partial sums go through global memory in two steps,
+// each counted -- every CTA publishes its n partial sums, one warp somewhere
+// adds those of a column, and everyone reads the n sums.
+// That costs a column about 5000 clocks more than one cluster's barrier and
+// sums, so it pays where the rows of 16 CTAs cost more than that.
+// Measured (us, one cluster or leaves -> every SM): 2304x64 619 -> 381,
+// 1024x128 1127 -> 796, 4096x128 2069 -> 966, 8192x128 2801 -> 1246,
+// 1620x180 2863 -> 1300, 8192x64 861 -> 498, three of 4096x128 2781 -> 1539.
+// Clusters of 8, summed first within the cluster and then over 15 to 19 of
+// them: 423, 776, 1010, 1362, 1602, 625, 1547.
 // ---------------------------------------------------------------------------
 constexpr int QRC_MAXT = 512;
 
@@ -315,18 +319,16 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
                                                          int lanes_log2) {
   extern __shared__ double qsm[];
   cg::cluster_group cluster = cg::this_cluster();
-  const int C = int(cluster.num_blocks());
-  const int rank = int(cluster.block_rank());
-  const int G = GRID ? q.G : 1;                // clusters per problem
-  const int pb = blockIdx.x / (C * G);
-  const int gid = GRID ? blockIdx.x / C - pb * G : 0;
+  const int C = GRID ? q.P : int(cluster.num_blocks());   // CTAs of a problem
+  const int pb = blockIdx.x / C;
+  const int rank = GRID ? blockIdx.x - pb * C : int(cluster.block_rank());
   const double* A = q.A.d(pb);
   double* const Qo = q.Q.d(pb);
   double* const Ro = q.R.n ? q.R.d(pb) : nullptr;
   const int m = q.m, n = q.n, k = min(m, n);
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-  const int chunk = (m + C * G - 1) / (C * G);
-  const int r0 = min(m, (gid * C + rank) * chunk), r1 = min(m, r0 + chunk), rows = r1 - r0;
+  const int chunk = (m + C - 1) / C;
+  const int r0 = min(m, rank * chunk), r1 = min(m, r0 + chunk), rows = r1 - r0;
   const int mcols = (k + C - 1) / C;        // columns of M solved here: rank, rank + C, ...
   double* part = qsm;                       // [2][n] my partial sums (read by every CTA)
   double* rowv = part + 2 * n;              // [2][n] row j of the matrix (in the row's owner)
@@ -340,9 +342,12 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
   double* mc = vs + k + 4;                  // [mcols][k] my columns of X_1^T, then of M (read by every CTA)
   double* tri = mc + mcols * k;             // packed columns: X^T X above the diagonal, then M
   double* W = tri + (tri_smem ? qr_tri(k) : 0);   // [n][ld], row i at i - r0
-  double* const gsum = GRID ? q.gsum + (long long)pb * 2 * G * n : nullptr;
+  double* const gpart = GRID ? q.gpart + (long long)pb * n * C : nullptr;
+  double* const gsum = GRID ? q.gsum + (long long)pb * n : nullptr;
   double* const grow = GRID ? q.grow + (long long)pb * 2 * n : nullptr;
-  bool live = true;                         // the polling thread: no wait has run out
+  unsigned* const cnt_part = GRID ? q.gcount + pb * 2 * QRG_LINE : nullptr;
+  unsigned* const cnt_sum = cnt_part + QRG_LINE;
+  bool live = true;                         // GRID: no wait of this thread has run out
   if (!GRID) {
     double* g = q.W + pb * q.wst + rank * (q.wst / C);
     if (!tri_smem) {
@@ -352,7 +357,7 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
     if (!w_smem) W = g;
   }
   auto cta_or_cluster_sync = [&]() {
-    if (C > 1)
+    if (!GRID && C > 1)
       cluster.sync();
     else
       __syncthreads();
@@ -391,7 +396,10 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
       }
       for (int o = L >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
       if (c < n && l == 0) {
-        part[b * n + c] = acc;
+        if (GRID)
+          __stcg(gpart + c * C + rank, acc);
+        else
+          part[b * n + c] = acc;
         if (own) {
           if (GRID)
             __stcg(grow + b * n + c, wc[jn]);
@@ -413,22 +421,32 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
     if (C > 2) s += __shfl_xor_sync(0xffffffffu, s, 2);
     return s + __shfl_xor_sync(0xffffffffu, s, 1);
   };
-  const int slice = (n + C - 1) / C;                  // GRID: columns whose sums over the cluster this CTA takes
-  const unsigned arrivals = unsigned(G * C) * unsigned((4 * slice + 31) / 32);   // warps that publish, per step
   pass(-1, 0, 0);
   for (int j = 0; j < k; ++j) {
     const int b = j & 1, owner = j / chunk;
     cta_or_cluster_sync();                            // column j: inner products and row j visible
     if (GRID) {
-      for (int t0 = tid - lane; t0 < 4 * slice; t0 += nt) {
-        const int ci = (t0 + lane) >> 2, l = lane & 3, c = rank * slice + ci;
-        const double s = cluster_sum(part + b * n + min(c, n - 1), l);
-        if (l == 0 && ci < slice && c < n) __stcg(gsum + (b * G + gid) * n + c, s);
+      // The next partial sums are written after these sums were awaited, the
+      // next sums after every CTA has arrived with new partial sums, row j
+      // alternates between two buffers: nothing is overwritten before its readers are done.
+      if (tid == 0) arrive_gpu(cnt_part);
+      for (int c = rank + (tid >> 5) * C; c < n; c += (nt >> 5) * C) {   // my columns, one warp each
+        if (lane == 0 && live) live = wait_arrivals(cnt_part, unsigned(j + 1) * C, q.flag);
         __syncwarp();
-        if (lane == 0) arrive_gpu(q.gcount + pb * QRG_LINE);
+        double v[QRG_MAXP / 32];
+#pragma unroll
+        for (int i = 0; i < QRG_MAXP / 32; ++i) v[i] = 32 * i + lane < C ? __ldcg(gpart + c * C + 32 * i + lane) : 0.0;
+        double s = v[0];
+#pragma unroll
+        for (int i = 1; i < QRG_MAXP / 32; ++i)
+          if (32 * i < C) s += v[i];
+        s = warp_sum(s);
+        if (lane == 0) {
+          __stcg(gsum + c, s);
+          arrive_gpu(cnt_sum);
+        }
       }
-      // both buffers are free again two steps on: an arrival follows its warp's reads
-      if (tid == nt - 32 && live) live = wait_arrivals(q.gcount + pb * QRG_LINE, unsigned(j + 1) * arrivals, q.flag);
+      if (tid == nt - 32 && live) live = wait_arrivals(cnt_sum, unsigned(j + 1) * n, q.flag);
       __syncthreads();
     }
     // row j, local copy: the threads that do not sum start at the far end
@@ -436,24 +454,17 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
       rowl[c] = GRID    ? __ldcg(grow + b * n + c)
                 : C > 1 ? *cluster.map_shared_rank(rowv + b * n + c, owner)
                         : rowv[b * n + c];
-    // sums over the CTAs (or clusters), four threads per column, column j first
-    for (int t0 = tid - lane; t0 < 4 * n; t0 += nt) {
-      const int ci = (t0 + lane) >> 2, l = lane & 3;
+    // sums over the CTAs, four threads per column (GRID: read by one), column j first
+    constexpr int SPREAD = GRID ? 0 : 2;
+    for (int t0 = tid - lane; t0 < n << SPREAD; t0 += nt) {
+      const int ci = (t0 + lane) >> SPREAD, l = lane & ((1 << SPREAD) - 1);
       int c = min(ci, n - 1) + j;
       if (c >= n) c -= n;
       double* slot = part + b * n + c;
       double alpha = 0.0, s;
       if (GRID) {
-        double v[QRG_MAX / 4];
-#pragma unroll
-        for (int i = 0; i < QRG_MAX / 4; ++i) v[i] = 4 * i + l < G ? __ldcg(gsum + (b * G + 4 * i + l) * n + c) : 0.0;
+        s = __ldcg(gsum + c);
         if (ci == 0) alpha = __ldcg(grow + b * n + j);
-        s = v[0];
-#pragma unroll
-        for (int i = 1; i < QRG_MAX / 4; ++i)
-          if (4 * i < G) s += v[i];
-        s += __shfl_xor_sync(0xffffffffu, s, 2);
-        s += __shfl_xor_sync(0xffffffffu, s, 1);
       } else if (C == 1) {
         s = *slot;
         if (ci == 0) alpha = rowv[b * n + j];
@@ -538,11 +549,26 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
       __syncwarp();
     }
   }
+  double* const gtri = GRID ? q.gtri + (long long)pb * qr_tri(k) : nullptr;
+  if (GRID) {
+    __syncthreads();
+    for (int c = rank + (tid >> 5) * C; c < k; c += (nt >> 5) * C)
+      for (int i = lane; i <= c; i += 32) __stcg(gtri + c * (c + 1) / 2 + i, mc[c / C * k + i]);
+  }
   cta_or_cluster_sync();                              // every column of M visible
-  for (int c = tid >> 5; c < k; c += nt >> 5) {
-    double* src = mc + (c / C) * k;
-    if (C > 1) src = cluster.map_shared_rank(src, c % C);
-    for (int i = lane; i <= c; i += 32) tri[c * (c + 1) / 2 + i] = src[i];
+  if (GRID) {
+    if (tid == 0) {
+      arrive_gpu(cnt_part);
+      if (live) wait_arrivals(cnt_part, unsigned(k + 1) * C, q.flag);
+    }
+    __syncthreads();
+    for (int i = tid; i < qr_tri(k); i += nt) tri[i] = __ldcg(gtri + i);
+  } else {
+    for (int c = tid >> 5; c < k; c += nt >> 5) {
+      double* src = mc + (c / C) * k;
+      if (C > 1) src = cluster.map_shared_rank(src, c % C);
+      for (int i = lane; i <= c; i += 32) tri[c * (c + 1) / 2 + i] = src[i];
+    }
   }
   __syncthreads();
   // Q = E - X M on my rows, one entry per thread at a time, lanes along rows
@@ -563,7 +589,7 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
     for (; a <= c; ++a) acc = fma(-x[a * ld], t[a], acc);
     Qo[(r0 + li) * q.qrs + c * q.qcs] = acc;
   }
-  if (C > 1) cluster.sync();   // no CTA leaves while others may still read its shared memory
+  if (!GRID && C > 1) cluster.sync();   // no CTA leaves while others may still read its shared memory
 }
 
 struct SvdArgs {
@@ -935,7 +961,7 @@ size_t qr_tri_bytes(int m, int n) { return sizeof(double) * size_t(qr_tri(std::m
 // A launch on clusters of c CTAs.
 struct ClusterLaunch {
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[2];
+  cudaLaunchAttribute at[1];
   ClusterLaunch(int ctas, int threads, size_t smem, int c, cudaStream_t st) {
     cfg.gridDim = dim3(ctas, 1, 1);
     cfg.blockDim = dim3(threads, 1, 1);
@@ -1069,43 +1095,32 @@ int tsqr_leaves(int m, int n, int np, double* clocks) {
   return best;
 }
 
-// How a matrix with m >= 1024 rows is factored: over G clusters of C CTAs at
-// once (G > 0), in L leaves (L > 0), or like any other.
+// How a matrix with m >= 1024 rows is factored: by P CTAs that are no cluster
+// (P > 0), in L leaves (L > 0), or like any other.
 struct TallPlan {
   int L = 0;
-  int C = 0, G = 0;
+  int P = 0;
   size_t bytes = 0;
 };
 
-// k_qr_cluster<true> on the shape with the least estimated time (G = 0: none):
-// qr_clocks' terms with the wait for the other clusters in every column (10500
-// clocks where one cluster has 5600; 1024x128 to 8192x128 come out within 15%,
-// 180 columns a quarter low).  Rows and triangle in shared memory, one CTA per
-// SM at most, and no more clusters than run at once.
+// k_qr_cluster<true> on every SM (P = 0: it does not fit, rows and triangle in
+// shared memory), with qr_clocks' terms and two waits for the other CTAs in a
+// column: 10500 clocks where one cluster has 5600 (the shapes above come out
+// within 15%).
 TallPlan qr_grid(int m, int n, int np, double* clocks) {
   TallPlan p;
   *clocks = 1e300;
   int dev = 0, sms = 0;
   PEPS_CUDA(cudaGetDevice(&dev));
   PEPS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const double warps = qr_threads(n) / 32;
-  for (int c = 4; c <= 16; c *= 2) {
-    int g = std::min(QRG_MAX, sms / c / np);
-    for (bool fits = false; g > 1 && !fits; g -= fits ? 0 : 1) {
-      const size_t b = qr_smem(m, n, c * g) - qr_head_bytes(m, n, c * g) + qr_head_bytes(m, n, c) + qr_tri_bytes(m, n);
-      fits = b <= kQrSmemMax && active_clusters(k_qr_cluster<true>, qr_threads(n), b, c) >= g * np;
-      if (!fits) continue;
-      const double rows = std::ceil(double(m) / (c * g));
-      const double step = 10500.0 + 180.0 * std::ceil(std::ceil(double(n) / c) / warps);
-      const double t = 14000.0 + n * (step + 24.0 * rows * 2.0 * n / 32.0 * (n < 64 ? 1.3 : 1.0));
-      if (t < *clocks) {
-        *clocks = t;
-        p.C = c;
-        p.G = g;
-        p.bytes = b;
-      }
-    }
-  }
+  const int c = std::min(QRG_MAXP, sms / np);
+  if (c < 2) return p;
+  const size_t b = qr_smem(m, n, c) + qr_tri_bytes(m, n);
+  if (b > kQrSmemMax || active_clusters(k_qr_cluster<true>, qr_threads(n), b, 1) < c * np) return p;
+  const double rows = std::ceil(double(m) / c);
+  *clocks = 14000.0 + n * (10500.0 + 24.0 * rows * 2.0 * n / 32.0 * (n < 64 ? 1.3 : 1.0));
+  p.P = c;
+  p.bytes = b;
   return p;
 }
 
@@ -1126,7 +1141,7 @@ TallPlan tall_plan(int m, int n, int np, bool whole) {
   if (whole) w = qr_grid(m, n, np, &grid);
   // the estimates are no better than a tenth
   if (!(p.L > 1 && leaves < 0.9 * direct)) p.L = 0;
-  if (w.G > 0 && grid < 0.9 * (p.L ? leaves : direct)) p = w;
+  if (w.P > 0 && grid < 0.9 * (p.L ? leaves : direct)) p = w;
   return cache.emplace(key, p).first->second;
 }
 
@@ -1190,10 +1205,10 @@ void qr_tsqr(Ctx& cx, int m, int n, int L, const TP& A, long long rs, long long 
   }
 }
 
-// One QR over G clusters.  Cooperative: its clusters wait for one another and
+// One QR on the whole device.  Cooperative: its CTAs wait for one another and
 // have to be resident together.
-void qr_clusters(Ctx& cx, int m, int n, const TallPlan& p, const TP& A, long long rs, long long cs, const TP& Q,
-                 long long qrs, long long qcs, const TP& R, int np) {
+void qr_whole(Ctx& cx, int m, int n, const TallPlan& p, const TP& A, long long rs, long long cs, const TP& Q,
+              long long qrs, long long qcs, const TP& R, int np) {
   QrArgs a;
   std::memset(static_cast<void*>(&a), 0, sizeof(a));
   a.m = m;
@@ -1205,21 +1220,22 @@ void qr_clusters(Ctx& cx, int m, int n, const TallPlan& p, const TP& A, long lon
   a.qrs = qrs;
   a.qcs = qcs;
   a.R = R.all(np);
-  a.G = p.G;
+  a.P = p.P;
   a.flag = cx.flag;
-  const size_t count = size_t(np) * QRG_LINE / 2, sums = size_t(np) * 2 * p.G * n, rows = size_t(np) * 2 * n;
-  double* w = cx.scratch(count + sums + rows);
+  const size_t b = size_t(np), count = b * QRG_LINE, part = b * n * p.P, tri = b * qr_tri(n);
+  double* w = cx.scratch(count + part + tri + b * 3 * n);
   a.gcount = reinterpret_cast<unsigned*>(w);
-  a.gsum = w + count;
-  a.grow = a.gsum + sums;
+  a.gpart = w + count;
+  a.gtri = a.gpart + part;
+  a.gsum = a.gtri + tri;
+  a.grow = a.gsum + b * n;
   PEPS_CUDA(cudaMemsetAsync(a.gcount, 0, count * sizeof(double), cx.st));
-  if (std::getenv("PEPS_VERBOSE")) std::fprintf(stderr, "[peps] qr %dx%d x%d: %d clusters of %d\n", m, n, np, p.G, p.C);
+  if (std::getenv("PEPS_VERBOSE")) std::fprintf(stderr, "[peps] qr %dx%d x%d: %d CTAs\n", m, n, np, p.P);
   Launch L(K_QR, cx.st, qr_flops(m, n) * np, 0);
-  ClusterLaunch c(p.C * p.G * np, qr_threads(n), p.bytes, p.C, cx.st);
-  c.at[1].id = cudaLaunchAttributeCooperative;
-  c.at[1].val.cooperative = 1;
-  c.cfg.numAttrs = 2;
-  PEPS_CUDA(cudaLaunchKernelEx(&c.cfg, k_qr_cluster<true>, a, 1, 1, qr_ld(m, p.C * p.G), qr_lanes_log2(n)));
+  int w_smem = 1, tri_smem = 1, ld = qr_ld(m, p.P), lanes = qr_lanes_log2(n);
+  void* args[] = {&a, &w_smem, &tri_smem, &ld, &lanes};
+  PEPS_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_qr_cluster<true>), dim3(p.P * np),
+                                        dim3(qr_threads(n)), args, p.bytes, cx.st));
   PEPS_CHECK_LAUNCH();
 }
 
@@ -1237,8 +1253,8 @@ void qr_thin(Ctx& cx, int m, int n, const TP& A, long long rs, long long cs, con
       qr_tsqr(cx, m, n, p.L, A, rs, cs, Q, qrs, qcs, R, np);
       return;
     }
-    if (p.G > 0) {
-      qr_clusters(cx, m, n, p, A, rs, cs, Q, qrs, qcs, R, np);
+    if (p.P > 0) {
+      qr_whole(cx, m, n, p, A, rs, cs, Q, qrs, qcs, R, np);
       return;
     }
   }

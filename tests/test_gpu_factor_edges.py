@@ -35,8 +35,8 @@ def test_norm_at_factor_edges(peps, Ly, Lx, D, chi, mode):
     assert abs(got[0] - want[0]) < 1e-10 and got[1] == want[1]
 
 
-# Boundary tensors of 1024 rows and more, whose QR is split over several
-# clusters: columns that are no multiple of a warp's or a cluster's share
+# Boundary tensors of 1024 rows and more, whose QR is split over every SM:
+# rows and columns that are no multiple of a warp's or a CTA's share
 # (1500x60), and more of them than four threads each cover (2240x140); just
 # below the rule, on one cluster (1008x63).  |ln N| is a few tens, and both
 # sides round in FP64 only: the 1e-10 above.
