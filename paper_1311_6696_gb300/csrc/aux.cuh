@@ -52,8 +52,9 @@ void finish_norm(Ctx& cx, const double* lns, int nl, const double* extra, const 
 void fill(Ctx& cx, const TP& x, long long n, double v);
 void copy(Ctx& cx, const TP& dst, const TP& src, long long n);
 
-// CU_0 separable boundaries of one oriented lattice (Section 5.1), computed
-// by one CTA.  Site tensors at `sites` (per-site offsets/dims in `meta`),
+// CU_0 separable boundaries of one oriented lattice (Section 5.1): the rows'
+// fixed parts in parallel and the fit on one cluster per lattice, or (D > 8, or
+// tables beyond shared memory) all of it on one CTA.  Site tensors at `sites` (per-site offsets/dims in `meta`),
 // closures as device matrices.  Output: out[r][x] = D x D matrix (stride
 // out_stride per row, mat_stride per site) on the up legs of row r, r = 1..Ly-1.
 struct Cu0Lattice {

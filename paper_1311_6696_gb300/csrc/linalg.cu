@@ -4,7 +4,8 @@
 // A matrix is split by rows over a thread-block cluster of 1-16 CTAs, kept in
 // shared memory where it fits, and the CTAs exchange partial sums through
 // distributed shared memory: the QR with one cluster barrier per Householder
-// column, the SVD with one per round of the round-robin Jacobi schedule.
+// column, the SVD with one per round of the round-robin Jacobi schedule.  A tall
+// QR that has the device to itself runs on every SM instead.
 #include <cooperative_groups.h>
 
 #include <algorithm>
