@@ -380,8 +380,10 @@ Layers layers(const MlpDims& m, const float* w) {
 constexpr int kMlpPrec = PEPS_PREC_BF16;
 
 // Activations H1, H2 of a forward pass: BF16 [n][W] in the layout of the next
-// layer's operand, biased, rectified and rounded by the GEMM that makes them
-// (the values an operand pack of the FP32 activations would make).
+// layer's operand, rows act_ld apart (16 bytes: W need not be a multiple of 8),
+// biased, rectified and rounded by the GEMM that makes them (the values an
+// operand pack of the FP32 activations would make).
+long long act_ld(const MlpDims& m) { return (m.W + 7) / 8 * 8; }
 size_t act_words(const MlpDims& m, long long n) {
   return tc_operand_words("bw,vw->bv", {int(n), m.W}, {m.W, m.W}, 1, kMlpPrec);
 }
@@ -402,6 +404,7 @@ void forward(Ctx& cx, const MlpDims& m, const float* w, const float* X, long lon
   c1.bias = L.b1;
   c1.relu = true;
   ein_tc(cx, "bi,wi->bw", X, 0, {nn, F}, L.W1, 0, {W, F}, TP(), 0, kMlpPrec, 1.0, TP(), nullptr, &c1);
+  PEPS_REQUIRE(o1.ld == act_ld(m), "internal: activation rows");
   c2.a_pre = &o1;
   c2.next = "bv,ov->bo";
   c2.next_bd = {o, W};
@@ -480,14 +483,15 @@ void loss_grad_buf(Ctx& cx, const MlpDims& m, const float* w, const float* X, co
   float* gb2 = gW2 + (long long)W * W;
   float* gW3 = gb2 + W;
   float* gb3 = gW3 + (long long)o * W;
-  // the activations are BF16 tensors [n][W]; what the rectifier held back is
-  // masked where the gradient is made
-  TcChain m2, m1;
+  // the activations are BF16 matrices [n][W] with padded rows; what the
+  // rectifier held back is masked where the gradient is made
+  TcChain m2, m1, act;
   m2.mask = H2;
   m1.mask = H1;
-  ein_tc(cx, "bo,bv->ov", dYo, 0, {nn, o}, H2, 2, {nn, W}, gW3, 0, kMlpPrec);
+  m2.mask_ld = m1.mask_ld = act.b_ld = act_ld(m);
+  ein_tc(cx, "bo,bv->ov", dYo, 0, {nn, o}, H2, 2, {nn, W}, gW3, 0, kMlpPrec, 1.0, TP(), nullptr, &act);
   ein_tc(cx, "bo,ov->bv", dYo, 0, {nn, o}, L.W3, 0, {o, W}, dH2, 0, kMlpPrec, 1.0, TP(), nullptr, &m2);
-  ein_tc(cx, "bv,bw->vw", dH2, 0, {nn, W}, H1, 2, {nn, W}, gW2, 0, kMlpPrec);
+  ein_tc(cx, "bv,bw->vw", dH2, 0, {nn, W}, H1, 2, {nn, W}, gW2, 0, kMlpPrec, 1.0, TP(), nullptr, &act);
   ein_tc(cx, "bv,vw->bw", dH2, 0, {nn, W}, L.W2, 0, {W, W}, dH1, 0, kMlpPrec, 1.0, TP(), nullptr, &m1);
   ein_tc(cx, "bw,bi->wi", dH1, 0, {nn, W}, X, 0, {nn, F}, gW1, 0, kMlpPrec);
   {

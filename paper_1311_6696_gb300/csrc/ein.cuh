@@ -153,7 +153,9 @@ struct TcOperand {
 // FP32 output of a plain call.
 //   bias:     added to every row of the result (one value per index of the N
 //             group), before relu (max with 0).
-//   mask:     BF16 tensor [M][N]; results where it is not positive become 0.
+//   mask:     BF16 tensor [M][N], rows mask_ld apart; results where it is not
+//             positive become 0.
+//   b_ld:     operand B has two indices, its rows b_ld elements apart (0: dense).
 struct TcChain {
   const TcOperand* a_pre = nullptr;
   const char* next = nullptr;
@@ -164,6 +166,8 @@ struct TcChain {
   const float* bias = nullptr;
   bool relu = false;
   const void* mask = nullptr;
+  long long mask_ld = 0;
+  long long b_ld = 0;
 };
 
 // Doubles a TcChain target needs for operand A of `spec` (hi and lo parts).

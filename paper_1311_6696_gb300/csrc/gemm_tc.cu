@@ -78,7 +78,8 @@ struct TcArgs {
   double alpha;
   int* flag;
   const float* bias;            // per column, or nullptr
-  const __nv_bfloat16* mask;    // [M][N], or nullptr
+  const __nv_bfloat16* mask;    // [M][N], rows mask_ld apart (a multiple of 8), or nullptr
+  long long mask_ld;
   int relu;
 };
 
@@ -86,7 +87,7 @@ struct TcArgs {
 __device__ __forceinline__ float finish_value(const TcArgs& g, long long m, long long n, float b, float v) {
   v += b;
   if (g.relu) v = fmaxf(v, 0.f);
-  if (g.mask && __bfloat162float(g.mask[m * g.N + n]) <= 0.f) v = 0.f;
+  if (g.mask && __bfloat162float(g.mask[m * g.mask_ld + n]) <= 0.f) v = 0.f;
   return v;
 }
 
@@ -261,9 +262,9 @@ __device__ __forceinline__ void put_run(const TcArgs& g, int pb, long long o, co
 // Bias, rectifier and mask on a lane's 16 scaled results of row m, columns n .. n + 15.
 __device__ __forceinline__ void finish_run(const TcArgs& g, long long m, long long n, const float* bias, float* v) {
   uint4 mk[2];
-  const bool vec = g.mask && g.N % 16 == 0 && m < g.M && n + 15 < g.N;
+  const bool vec = g.mask && m < g.M && n + 15 < g.N;   // n is a multiple of 16: aligned
   if (vec) {
-    const uint4* src = reinterpret_cast<const uint4*>(g.mask + m * g.N + n);
+    const uint4* src = reinterpret_cast<const uint4*>(g.mask + m * g.mask_ld + n);
     mk[0] = src[0];
     mk[1] = src[1];
   }
@@ -275,7 +276,7 @@ __device__ __forceinline__ void finish_run(const TcArgs& g, long long m, long lo
     if (vec) {
       if (__bfloat162float(mh[j]) <= 0.f) v[j] = 0.f;
     } else if (g.mask && m < g.M && n + j < g.N) {
-      if (__bfloat162float(g.mask[m * g.N + n + j]) <= 0.f) v[j] = 0.f;
+      if (__bfloat162float(g.mask[m * g.mask_ld + n + j]) <= 0.f) v[j] = 0.f;
     }
   }
 }
@@ -996,8 +997,12 @@ struct Operand {
 // `rowletters`, K over `kletters`; problem p at rows p * pad ..).
 Operand pack(Ctx& cx, const TP& src, int np, long long pad, int src_f64, const std::string& letters,
              const Dims& dims, const std::string& rowletters, const std::string& kletters, int bf16, int split,
-             double* mem) {
+             double* mem, long long src_ld = 0) {
   auto st = strides_of(dims);
+  if (src_ld) {   // a matrix with its rows src_ld apart
+    PEPS_REQUIRE(dims.size() == 2 && src_ld >= dims[1], "internal: row pitch");
+    st[0] = src_ld;
+  }
   PackArgs p;
   std::memset(static_cast<void*>(&p), 0, sizeof(p));
   Operand o;
@@ -1301,7 +1306,7 @@ void ein_tc(Ctx& cx, const char* spec, const TP& A, int a_f64, const Dims& ad, c
   Operand ob;
   if (!cached || fresh) {
     ob = pack(cx, B, np, pad_n, b_f64, p.b, bd, nL, kL, bf16, split,
-              cached ? static_cast<double*>(cached->hi) : mem + wa);
+              cached ? static_cast<double*>(cached->hi) : mem + wa, chain ? chain->b_ld : 0);
     if (cached) cached->ld = ob.ld;
   } else {
     ob.hi = cached->hi;
@@ -1401,6 +1406,9 @@ void ein_tc(Ctx& cx, const char* spec, const TP& A, int a_f64, const Dims& ad, c
     PEPS_REQUIRE(np == 1, "internal: bias or mask with several problems");
     g.bias = chain->bias;
     g.mask = static_cast<const __nv_bfloat16*>(chain->mask);
+    g.mask_ld = chain->mask_ld;
+    PEPS_REQUIRE(!g.mask || (g.mask_ld >= N && g.mask_ld % 8 == 0 && (reinterpret_cast<uintptr_t>(g.mask) & 15) == 0),
+                 "internal: mask rows");
     g.relu = chain->relu ? 1 : 0;
   }
   const double flops = 2.0 * double(M) * double(N) * double(K) * np;

@@ -185,3 +185,26 @@ def test_gradient_and_inference_at_batch_edges(env, D, n):
     assert abs(loss - want_loss) < 1e-2 * abs(want_loss)
     assert _rel(grad.cpu().double().numpy(), want.numpy()) < 1e-2
     assert np.max(np.abs(peps.mlp_predict(w, X.cuda(), 2, D).cpu().double().numpy() - sig.numpy())) < 1e-3
+
+
+@pytest.mark.parametrize("W,n", [(16, 130), (20, 300), (33, 129), (250, 300), (260, 257)])
+def test_gradient_at_widths_that_are_no_multiple_of_eight(env, W, n):
+    """Activations are kept with their rows padded to 16 bytes; every width is
+    accepted.  Reference and tolerance as above, batches beyond one tile's rows."""
+    torch, peps = env
+    D, F = 3, 2 * 3 ** 4 + 2 * 9
+    g = torch.Generator().manual_seed(11 * W + n)
+    low = torch.tril(0.2 * torch.randn(n, D, D, generator=g, dtype=torch.float64), -1) + torch.eye(D, dtype=torch.float64)
+    low = low / (low @ low.mT).square().sum((1, 2), keepdim=True).sqrt().sqrt()
+    site = torch.randn(n, 2 * D ** 4, generator=g, dtype=torch.float64)
+    X = torch.cat([site / site.norm(dim=1, keepdim=True), (low @ low.mT).reshape(n, -1), low.reshape(n, -1)], 1).float()
+    Y = torch.eye(D).reshape(1, -1).repeat(n, 1) / D ** 0.5
+    w = peps.mlp_init(2, D, W, seed=D)
+    k = W * F + W + W * W + W
+    w[k:] = 0.05 * torch.randn(D * D * W + D * D, generator=g).cuda()
+    w[W * F:W * F + W] = 0.1 * torch.randn(W, generator=g).cuda()
+    loss, grad = peps.mlp_loss_grad(w, X.cuda(), Y.cuda(), 2, D, W)
+    want_loss, want, sig = _network_with_bf16_operands(torch, w.cpu(), X, Y, F, W, D)
+    assert abs(loss - want_loss) < 1e-2 * abs(want_loss)
+    assert _rel(grad.cpu().double().numpy(), want.numpy()) < 1e-2
+    assert np.max(np.abs(peps.mlp_predict(w, X.cuda(), 2, D, W).cpu().double().numpy() - sig.numpy())) < 1e-3
