@@ -771,7 +771,7 @@ OLat sub(const OLat& f, int r0, int r1, int c0, int c1) {
   return s;
 }
 
-// CU_0 separable boundaries from all four sides (one CTA per side): sig[o] is
+// CU_0 separable boundaries from all four sides: sig[o] is
 // [L_o][W_o][D*D], matrix (r, x) on the up legs of row r of orientation o.
 void cu0_all_sides(Ctx& cx, const peps_lattice* lat, Oriented& ori, Arena& keep, double* sig[4]) {
   const int Ly = lat->Ly, Lx = lat->Lx, d = lat->d, D = lat->D, DM2 = D * D;
@@ -807,7 +807,7 @@ void cu0_all_sides(Ctx& cx, const peps_lattice* lat, Oriented& ori, Arena& keep,
     q.left = closure_ones;
     q.right = closure_ones;
     q.out = sig[o];
-    q.work = cx.ws->dalloc(cu0_work_size(L.Lx, d, D));
+    q.work = nullptr;
     q.max_half = std::max(1, cx.cu0_cap);
     q.tol = 1e-13;
   }

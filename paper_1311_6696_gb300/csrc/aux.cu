@@ -993,14 +993,9 @@ void copy(Ctx& cx, const TP& dst, const TP& src, long long n) {
   PEPS_CHECK_LAUNCH();
 }
 
-size_t cu0_work_size(int Lx, int d, int Dmax) {
-  const size_t D2 = size_t(Dmax) * Dmax, T = size_t(tri_count(Dmax));
-  if (cu0_fast(Lx, d, Dmax)) return 2 * size_t(Lx) * T * T * T;
-  return 2 * size_t(d) * D2 * D2 + 2 * size_t(Lx) * D2 + D2;
-}
-
-void cu0_launch(Ctx& cx, const Cu0Lattice* lats, int nlat) {
-  auto* dev = static_cast<const Cu0Lattice*>(stage(cx, lats, sizeof(Cu0Lattice) * nlat));
+// All lattices of a call run on the kernels that every one of them fits, and
+// the workspaces are laid out for those.
+void cu0_launch(Ctx& cx, Cu0Lattice* lats, int nlat) {
   int Ly = 1, Lx = 1, D = 1, d = 1;
   bool fast = true;
   for (int i = 0; i < nlat; ++i) {
@@ -1010,6 +1005,11 @@ void cu0_launch(Ctx& cx, const Cu0Lattice* lats, int nlat) {
     d = std::max(d, lats[i].d);
     fast = fast && cu0_fast(lats[i].Lx, lats[i].d, lats[i].Dmax);
   }
+  for (int i = 0; i < nlat; ++i) {
+    const size_t x = lats[i].Lx, D2 = size_t(lats[i].Dmax) * lats[i].Dmax, T = tri_count(lats[i].Dmax);
+    lats[i].work = cx.ws->dalloc(fast ? 2 * x * T * T * T : 2 * lats[i].d * D2 * D2 + 2 * x * D2 + D2);
+  }
+  auto* dev = static_cast<const Cu0Lattice*>(stage(cx, lats, sizeof(Cu0Lattice) * nlat));
   Launch L(K_CU0, cx.st);
   if (!fast) {   // D > 8, or rows too long for shared memory: one CTA per side
     k_cu0<<<nlat, 256, 0, cx.st>>>(dev, cx.flag);

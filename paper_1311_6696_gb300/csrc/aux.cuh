@@ -66,11 +66,10 @@ struct Cu0Lattice {
   const double* left;           // [Ly] closures, stride Dmax^2
   const double* right;          // [Ly]
   double* out;                  // [Ly][Lx][Dmax^2]
-  double* work;                 // scratch, see cu0_work_size
+  double* work;                 // set by cu0_launch
   int max_half;
   double tol;
 };
-size_t cu0_work_size(int Lx, int d, int Dmax);
-void cu0_launch(Ctx& cx, const Cu0Lattice* lats, int nlat);
+void cu0_launch(Ctx& cx, Cu0Lattice* lats, int nlat);
 
 }  // namespace peps

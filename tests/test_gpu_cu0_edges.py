@@ -33,3 +33,14 @@ def test_cluster_environments_at_cu0_edges(peps, Ly, Lx, D, n):
             continue
         g, w = got.expect(kind, op).ravel(), np.asarray(O.expect_all(want, kind, op), dtype=float).ravel()
         assert np.max(np.abs(g - w) / np.maximum(np.abs(w), 1e-2)) < 1e-10, kind
+
+
+# Rows too long for shared memory beside columns of one or two sites: all four
+# sides take the kernel that the long ones need.
+@pytest.mark.parametrize("Ly,Lx,D", [(1, 2600, 2), (2570, 1, 2), (1, 1300, 3), (1, 800, 4)])
+def test_long_thin_lattices(peps, Ly, Lx, D):
+    from paper_1311_6696_gb300 import synth
+    A = synth.peps_gauss(Ly, Lx, 2, D, seed=60 + D)
+    got = peps.env_cluster(A, 1, chi=D * D, mode="var").expect("site", O.SZ).ravel()
+    want = np.asarray(O.expect_all(O.env_cluster(A, 1, chi=D * D, mode="var"), "site", O.SZ), dtype=float).ravel()
+    assert np.max(np.abs(got - want) / np.maximum(np.abs(want), 1e-2)) < 1e-10
