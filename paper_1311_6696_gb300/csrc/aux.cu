@@ -609,6 +609,9 @@ constexpr int CU0_MAXD = 8;
 constexpr int CU0_MAXT = CU0_MAXD * (CU0_MAXD + 1) / 2;
 constexpr int CU0_THREADS = 256;
 
+// 2^k for |k| <= 1022.
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+
 __host__ __device__ inline int tri_count(int n) { return n * (n + 1) / 2; }
 
 // pi <= pj of packed pair p = pj (pj + 1) / 2 + pi, the same for every dimension.
@@ -626,6 +629,7 @@ __device__ __forceinline__ void pair_tables(int* pi, int* pj) {
 __global__ void __launch_bounds__(CU0_THREADS) k_cu0_build(const Cu0Lattice* lats, int r, int parts) {
   extern __shared__ double bsm[];
   __shared__ int pi[CU0_MAXT], pj[CU0_MAXT];
+  __shared__ unsigned s_top;
   const Cu0Lattice L = lats[blockIdx.y];
   const int x = blockIdx.x / parts, part = blockIdx.x % parts;
   if (r + 1 >= L.Ly || x >= L.Lx) return;
@@ -637,8 +641,25 @@ __global__ void __launch_bounds__(CU0_THREADS) k_cu0_build(const Cu0Lattice* lat
   double* A = bsm;              // [s][u][l][n][r]
   double* B = bsm + K * P3;     // [s][v][l][n][r] = sum_u S[u,v] A
   pair_tables(pi, pj);
-  for (int e = tid; e < K * P3; e += nt) A[e] = Ag[e];
+  if (tid == 0) s_top = 0;
   __syncthreads();
+  // The matrices do not depend on the site's scale, but an environment's norm
+  // is formed from its eighth power: a site far from order one is brought
+  // there by an exact power of two.
+  unsigned top = 0;
+  for (int e = tid; e < K * P3; e += nt) {
+    const double v = Ag[e];
+    A[e] = v;
+    top = max(top, unsigned(__double2hiint(v)) & 0x7fffffffu);
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if ((tid & 31) == 0) atomicMax(&s_top, top);
+  __syncthreads();
+  const int shift = min(1022, max(-1022, 1023 - int(s_top >> 20)));
+  if (abs(shift) > 64) {
+    for (int e = tid; e < K * P3; e += nt) A[e] *= pow2(shift);
+    __syncthreads();
+  }
   for (int e = tid; e < K * P3; e += nt) {
     const int sv = e / P3, o = e - sv * P3, s = sv / du, v = sv - s * du;
     const double* a = A + s * du * P3 + o;
