@@ -609,9 +609,6 @@ constexpr int CU0_MAXD = 8;
 constexpr int CU0_MAXT = CU0_MAXD * (CU0_MAXD + 1) / 2;
 constexpr int CU0_THREADS = 256;
 
-// 2^k for |k| <= 1022.
-__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
-
 __host__ __device__ inline int tri_count(int n) { return n * (n + 1) / 2; }
 
 // pi <= pj of packed pair p = pj (pj + 1) / 2 + pi, the same for every dimension.
@@ -650,13 +647,13 @@ __global__ void __launch_bounds__(CU0_THREADS) k_cu0_build(const Cu0Lattice* lat
   for (int e = tid; e < K * P3; e += nt) {
     const double v = Ag[e];
     A[e] = v;
-    top = max(top, unsigned(__double2hiint(v)) & 0x7fffffffu);
+    top = max(top, high_word(v));
   }
   top = __reduce_max_sync(0xffffffffu, top);
   if ((tid & 31) == 0) atomicMax(&s_top, top);
   __syncthreads();
-  const int shift = min(1022, max(-1022, 1023 - int(s_top >> 20)));
-  if (abs(shift) > 64) {
+  const int shift = order_one(s_top);
+  if (shift != 0) {
     for (int e = tid; e < K * P3; e += nt) A[e] *= pow2(shift);
     __syncthreads();
   }

@@ -698,13 +698,21 @@ __global__ void __launch_bounds__(SVC_MAXT) k_svd_cluster(const SvdArgs s, int h
   double* nrm = tb + npair;                   // [q]
   int* order = reinterpret_cast<int*>(nrm + q);   // [q]
   __shared__ int s_rot;
+  __shared__ unsigned s_top, s_all;
   double* G = rows_smem ? ssm + svd_head(q) : work + (head_smem ? 0 : svd_head(q));
   const double* A = s.A.d(pb);
   const bool rows_first = s.rs < s.cs;
+  if (tid == 0) s_top = s_all = 0;
+  __syncthreads();
+  unsigned top = 0;
   for (long long e = tid; e < (long long)gr * q; e += nt) {
     const int j = int(rows_first ? e / gr : e % q), li = int(rows_first ? e % gr : e / q);
-    G[(long long)j * ld + li] = A[(g0 + li) * s.rs + j * s.cs];
+    const double v = A[(g0 + li) * s.rs + j * s.cs];
+    G[(long long)j * ld + li] = v;
+    top = max(top, high_word(v));
   }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (lane == 0) atomicMax(&s_top, top);
   for (int j = warp; j < q; j += nw)
     for (int li = lane; li < vr; li += 32) G[(long long)j * ld + cp + li] = (v0 + li == j) ? 1.0 : 0.0;
   for (int j = tid; j < q; j += nt) {
@@ -718,6 +726,17 @@ __global__ void __launch_bounds__(SVC_MAXT) k_svd_cluster(const SvdArgs s, int h
       __syncthreads();
   };
   auto sum_parts = [&](double* slot) { return C > 1 ? remote_sum(cluster, slot, C) : *slot; };
+  // A matrix far from order one is brought there by an exact power of two (and
+  // its singular values back): the norms are squares and the rotation test
+  // compares their products.
+  cta_or_cluster_sync();
+  if (tid < C) atomicMax(&s_all, C > 1 ? *cluster.map_shared_rank(&s_top, tid) : s_top);
+  __syncthreads();
+  const int shift = order_one(s_all);
+  if (shift != 0)
+    for (int j = warp; j < q; j += nw)
+      for (int li = lane; li < gr; li += 32) G[(long long)j * ld + li] *= pow2(shift);
+  const double unscale = pow2(-shift);
   // the scales into the columns (after a barrier; followed by one)
   auto rescale = [&]() {
     for (int j = warp; j < q; j += nw) {
@@ -785,12 +804,16 @@ __global__ void __launch_bounds__(SVC_MAXT) k_svd_cluster(const SvdArgs s, int h
         if (b < q) {
           const double da = ds[a], db = ds[b], A2 = al[a], B2 = al[b];
           const double ga = sum_parts(part + buf * 2 * npair + pr) * da * db;
-          // gamma^2 > tol^2 alpha beta, tested on the sign of the difference
-          const double over = fma(-(tol * A2), tol * B2, ga * ga);
-          if (__double2hiint(over) > 0 || (__double2hiint(over) == 0 && __double2loint(over) != 0)) {
-            const double dl = B2 - A2;
-            const int k = 1023 - ((max(__double2hiint(A2), __double2hiint(B2)) >> 20) & 0x7ff);
-            const float df = float(scale2(dl, k)), gf = 2.f * float(scale2(ga, k));
+          // gamma^2 > tol^2 alpha beta, tested on the sign of the difference,
+          // everything scaled by the larger norm's exponent (fourth powers of
+          // a small column would underflow); no rotation where a norm is no
+          // finite number
+          const double dl = B2 - A2;
+          const int k = 1023 - ((max(__double2hiint(A2), __double2hiint(B2)) >> 20) & 0x7ff);
+          const double g1 = scale2(ga, k);
+          const double over = fma(-(tol * scale2(A2, k)), tol * scale2(B2, k), g1 * g1);
+          if (k > -1024 && (__double2hiint(over) > 0 || (__double2hiint(over) == 0 && __double2loint(over) != 0))) {
+            const float df = float(scale2(dl, k)), gf = 2.f * float(g1);
             double t;
             if (fabsf(gf) > 1e-18f) {
               const float h = fabsf(df) + sqrtf(fmaf(df, df, gf * gf));
@@ -866,7 +889,7 @@ __global__ void __launch_bounds__(SVC_MAXT) k_svd_cluster(const SvdArgs s, int h
     // US[i][r] = G(i, order[r]) for my G rows; Vt[r][j] = V(j, order[r]) for my V rows
     for (int e = tid; e < gr * kk; e += nt) {
       const int li = e / kk, r = e % kk;
-      US[(long long)(g0 + li) * kk + r] = (r < q) ? G[(long long)order[r] * ld + li] : 0.0;
+      US[(long long)(g0 + li) * kk + r] = (r < q) ? G[(long long)order[r] * ld + li] * unscale : 0.0;
     }
     for (int e = tid; e < vr * kk; e += nt) {
       const int r = e / vr, li = e % vr;
@@ -876,7 +899,7 @@ __global__ void __launch_bounds__(SVC_MAXT) k_svd_cluster(const SvdArgs s, int h
     // US[i][r] = V(i, order[r]) * nrm for my V rows; Vt[r][j] = G(j, order[r]) / nrm for my G rows
     for (int e = tid; e < vr * kk; e += nt) {
       const int li = e / kk, r = e % kk;
-      US[(long long)(v0 + li) * kk + r] = (r < q) ? G[(long long)order[r] * ld + cp + li] * nrm[order[r]] : 0.0;
+      US[(long long)(v0 + li) * kk + r] = (r < q) ? G[(long long)order[r] * ld + cp + li] * (nrm[order[r]] * unscale) : 0.0;
     }
     for (int e = tid; e < gr * kk; e += nt) {
       const int r = e / gr, li = e % gr;

@@ -10,6 +10,21 @@ constexpr int FLAG_CU0_NOCONV = 2;
 constexpr int FLAG_BAD_VALUE = 4;
 constexpr int FLAG_TIMEOUT = 8;
 
+#ifdef __CUDACC__
+// 2^k for |k| <= 1022.
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+
+// k such that 2^k brings a tensor to order one, from the high word of its
+// largest entry (sign bit clear).  0 within 2^+-64, where the squares and
+// fourth powers that the kernels form have room.
+__device__ __forceinline__ int order_one(unsigned top) {
+  const int k = min(1022, max(-1022, 1023 - int(top >> 20)));
+  return abs(k) > 64 ? k : 0;
+}
+
+__device__ __forceinline__ unsigned high_word(double v) { return unsigned(__double2hiint(v)) & 0x7fffffffu; }
+#endif
+
 // Thin QR of the m x n matrix with element (i,j) at A[i*rs + j*cs], for each
 // problem of the pointer sets.  Writes Q (m x k, k = min(m,n)) to
 // Q[i*qrs + j*qcs] and, if R is present, R (k x n) row-major.  Householder

@@ -43,3 +43,22 @@ def test_separable_boundaries_do_not_depend_on_the_scale(peps, D, k):
     a = peps.env_cluster(A, 1, chi=D * D, mode="var")
     b = peps.env_cluster(A * 2.0 ** -k, 1, chi=D * D, mode="var")
     assert np.max(np.abs(a.expect("site", O.SZ) - b.expect("site", O.SZ))) < 1e-12
+
+
+# A row of 6 sites scales by 2^(-12 k), to 1e-137 (and to 1e137) before it is
+# rescaled; fewer columns than the SVD's preconditioning takes (D = 2, chi = 2),
+# more of them (D = 3), and the variational fit, whose local tensors carry the
+# row's scale as well.
+@pytest.mark.parametrize("D,chi,mode", [(2, 2, "svd"), (3, 4, "svd"), (3, 6, "var")])
+@pytest.mark.parametrize("k", [10, 22, 38, -38])
+def test_full_environments_do_not_depend_on_the_scale(peps, D, chi, mode, k):
+    Ly, Lx = 4, 6
+    A = _lattice(Ly, Lx, D, seed=70 + D)
+    B = A * 2.0 ** -k
+    shift = -2.0 * k * math.log(2.0) * Ly * Lx
+    ln, sign = peps.norm(A, chi, mode=mode, seed=2)
+    ln_b, sign_b = peps.norm(B, chi, mode=mode, seed=2)
+    assert abs(ln_b - ln - shift) < 1e-10 and sign_b == sign
+    a, b = peps.env_full(A, chi, mode=mode, seed=2), peps.env_full(B, chi, mode=mode, seed=2)
+    for kind, op in (("site", O.SZ), ("hbond", O.SDOTS), ("vbond", O.SDOTS)):
+        assert np.max(np.abs(a.expect(kind, op) - b.expect(kind, op))) < 1e-12, kind
