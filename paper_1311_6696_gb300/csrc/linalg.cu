@@ -69,7 +69,8 @@ struct QrArgs {
   double* gsum;      // [n] their sums
   double* grow;      // [2][n] row j of the matrix
   double* gtri;      // M, packed columns
-  unsigned* gcount;  // two counters QRG_LINE apart, zero at launch: partial sums, sums
+  unsigned* gcount;  // four words QRG_LINE apart, zero at launch: arrivals with partial sums, with sums and with
+                     // the largest high word, and that word
   int* flag;
 };
 constexpr int QRG_LINE = 32;    // 128 bytes
@@ -346,8 +347,11 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
   double* const gpart = GRID ? q.gpart + (long long)pb * n * C : nullptr;
   double* const gsum = GRID ? q.gsum + (long long)pb * n : nullptr;
   double* const grow = GRID ? q.grow + (long long)pb * 2 * n : nullptr;
-  unsigned* const cnt_part = GRID ? q.gcount + pb * 2 * QRG_LINE : nullptr;
+  unsigned* const cnt_part = GRID ? q.gcount + pb * 4 * QRG_LINE : nullptr;
   unsigned* const cnt_sum = cnt_part + QRG_LINE;
+  unsigned* const cnt_top = cnt_sum + QRG_LINE;
+  unsigned* const gtop = cnt_top + QRG_LINE;
+  __shared__ unsigned s_warp[QRC_MAXT / 32], s_top;   // largest high word of a warp's loads, of my rows (read by every CTA)
   bool live = true;                         // GRID: no wait of this thread has run out
   if (!GRID) {
     double* g = q.W + pb * q.wst + rank * (q.wst / C);
@@ -363,18 +367,50 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
     else
       __syncthreads();
   };
+  unsigned top = 0;
   if (q.cs == 1) {
     for (int e = tid; e < rows * n; e += nt) {
       const int li = e / n, j = e - li * n;
-      W[j * ld + li] = A[(r0 + li) * q.rs + j];
+      const double v = A[(r0 + li) * q.rs + j];
+      W[j * ld + li] = v;
+      top = max(top, high_word(v));
     }
   } else {
     for (int e = tid; e < rows * n; e += nt) {
       const int j = e / rows, li = e - j * rows;
-      W[j * ld + li] = A[(r0 + li) * q.rs + j * q.cs];
+      const double v = A[(r0 + li) * q.rs + j * q.cs];
+      W[j * ld + li] = v;
+      top = max(top, high_word(v));
     }
   }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (lane == 0) s_warp[tid >> 5] = top;
   __syncthreads();
+  // A matrix far from order one is brought there by an exact power of two (and
+  // R back): a column whose squares underflow would get no reflector.
+  top = __reduce_max_sync(0xffffffffu, lane < nt >> 5 ? s_warp[lane] : 0u);
+  if (GRID) {
+    if (tid == 0) {
+      atomicMax(gtop, top);
+      arrive_gpu(cnt_top);
+      live = wait_arrivals(cnt_top, unsigned(C), q.flag);
+      s_top = __ldcg(gtop);
+    }
+    __syncthreads();
+    top = s_top;
+  } else if (C > 1) {
+    if (tid == 0) s_top = top;
+    cluster.sync();
+    top = __reduce_max_sync(0xffffffffu, lane < C ? *cluster.map_shared_rank(&s_top, lane) : 0u);
+  }
+  const int shift = order_one(top);                   // the same in every CTA
+  if (shift != 0) {
+    for (int e = tid; e < rows * n; e += nt) {
+      const int c = e / rows, li = e - c * rows;
+      W[c * ld + li] *= pow2(shift);
+    }
+    __syncthreads();
+  }
   // One pass over the columns: the update with reflector column j (w from
   // wfin; j < 0: none) for c > jn, then the inner products with column jn
   // (final already) over rows >= jn for c > jn, over rows > jn otherwise.  The
@@ -524,7 +560,9 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
   if (Ro) {
     for (int e = tid; e < rows * n; e += nt) {
       const int li = e / n, j = e - li * n, i = r0 + li;
-      if (i < k) Ro[(long long)i * n + j] = (j >= i) ? W[j * ld + li] : 0.0;
+      if (i >= k) continue;
+      const double v = (j >= i) ? W[j * ld + li] : 0.0;
+      Ro[(long long)i * n + j] = shift != 0 ? v * pow2(-shift) : v;
     }
   }
   for (int j = tid; j < k; j += nt) vs[j] = vs[j] + nb[j];
@@ -1246,7 +1284,7 @@ void qr_whole(Ctx& cx, int m, int n, const TallPlan& p, const TP& A, long long r
   a.R = R.all(np);
   a.P = p.P;
   a.flag = cx.flag;
-  const size_t b = size_t(np), count = b * QRG_LINE, part = b * n * p.P, tri = b * qr_tri(n);
+  const size_t b = size_t(np), count = b * 2 * QRG_LINE, part = b * n * p.P, tri = b * qr_tri(n);
   double* w = cx.scratch(count + part + tri + b * 3 * n);
   a.gcount = reinterpret_cast<unsigned*>(w);
   a.gpart = w + count;

@@ -62,3 +62,14 @@ def test_full_environments_do_not_depend_on_the_scale(peps, D, chi, mode, k):
     a, b = peps.env_full(A, chi, mode=mode, seed=2), peps.env_full(B, chi, mode=mode, seed=2)
     for kind, op in (("site", O.SZ), ("hbond", O.SDOTS), ("vbond", O.SDOTS)):
         assert np.max(np.abs(a.expect(kind, op) - b.expect(kind, op))) < 1e-12, kind
+
+
+# Rows down to 1e-148: the local tensors' smaller columns lie below the square
+# root of the smallest double, their QR's squares beyond its range.
+@pytest.mark.parametrize("D,chi,mode", [(2, 2, "svd"), (3, 4, "svd"), (3, 6, "var"), (4, 5, "var")])
+def test_norm_near_the_end_of_the_range(peps, D, chi, mode):
+    Ly, Lx, k = 3, 6, 41
+    A = _lattice(Ly, Lx, D, seed=90 + D)
+    ln, sign = peps.norm(A, chi, mode=mode, seed=2)
+    ln_b, sign_b = peps.norm(A * 2.0 ** -k, chi, mode=mode, seed=2)
+    assert abs(ln_b - ln + 2.0 * k * math.log(2.0) * Ly * Lx) < 1e-10 and sign_b == sign
