@@ -58,8 +58,8 @@ struct QrArgs {
   TP Q;
   long long qrs, qcs;
   TP R;         // absent: R not wanted
-  double* W;    // work per problem (problem p at W + p * wst): k_qr_cluster's rows where they
-                // do not fit in shared memory (C * ld * n), k_qr_house's m x n copy
+  double* W;    // work per problem (problem p at W + p * wst): what k_qr_cluster's shared memory
+                // does not hold (wst / C per CTA), k_qr_house's m x n copy
   double* Qw;   // k_qr_house: m*k work per problem, column-major (+ p * qst)
   double* tau;  // k_qr_house: k per problem (+ p * tst)
   long long wst, qst, tst;
@@ -213,7 +213,12 @@ __device__ __forceinline__ double remote_sum(cg::cluster_group& cl, double* slot
 // 824 -> 618, 1620x180 3637 -> 2861, 8192x128 (tall-skinny, four leaves)
 // 3847 -> 2853; 16 of 36x36 270 -> 123 (those ran in global memory, one CTA
 // each).  Orthogonality stays at 1e-15 to 7e-15; |A - QR| is 1 to 3 eps of a
-// column's norm.
+// column's norm.  Shared memory holds the sums (88 bytes a column, to 2600
+// columns), then the rows, M's columns and the triangle, each while it fits; the
+// rest lies in global memory.  With M's columns in shared memory or nowhere,
+// squares of more than 400 columns kept their rows in global memory and more
+// than 592 columns ran on one CTA: 448x448 52.3 -> 7.3 ms, 640x600 120 -> 15.7,
+// 1024x1024 475 -> 58.9, 9600x640 3009 -> 141.
 //
 // GRID: the rows of one matrix over every SM.  One cluster has 16 SMs, and of
 // clusters of 16 only seven run at once, so that one matrix, or its leaves,
@@ -231,10 +236,10 @@ __device__ __forceinline__ double remote_sum(cg::cluster_group& cl, double* slot
 // ---------------------------------------------------------------------------
 constexpr int QRC_MAXT = 512;
 
-// Per-CTA shared memory besides the rows and the triangle, in doubles.
-__host__ __device__ inline long long qr_head(int n, int k, int c) {
-  return 7LL * n + 4LL * k + 4 + (long long)((k + c - 1) / c) * k;
-}
+// Per-CTA shared memory besides the rows, the columns of M and the triangle, in doubles.
+__host__ __device__ inline long long qr_head(int n, int k) { return 7LL * n + 4LL * k + 4; }
+// A CTA's columns of M.
+__host__ __device__ inline long long qr_mc(int k, int c) { return (long long)((k + c - 1) / c) * k; }
 // The triangle: X^T X, then M.
 __host__ __device__ inline long long qr_tri(int k) { return (long long)k * (k + 1) / 2; }
 
@@ -317,8 +322,8 @@ __device__ __forceinline__ bool wait_arrivals(const unsigned* p, unsigned target
 // are enough to keep the FP64 pipe busy, and each doubling adds an addition to
 // every sum.
 template <bool GRID>
-__global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_smem, int tri_smem, int ld,
-                                                         int lanes_log2) {
+__global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_smem, int mc_smem, int tri_smem,
+                                                         int ld, int lanes_log2) {
   extern __shared__ double qsm[];
   cg::cluster_group cluster = cg::this_cluster();
   const int C = GRID ? q.P : int(cluster.num_blocks());   // CTAs of a problem
@@ -342,7 +347,7 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
   double* nb = gs + k;                      // [k] -beta
   double* vs = nb + k;                      // [k] alpha - beta
   double* mc = vs + k + 4;                  // [mcols][k] my columns of X_1^T, then of M (read by every CTA)
-  double* tri = mc + mcols * k;             // packed columns: X^T X above the diagonal, then M
+  double* tri = mc + (mc_smem ? qr_mc(k, C) : 0); // packed columns: X^T X above the diagonal, then M
   double* W = tri + (tri_smem ? qr_tri(k) : 0);   // [n][ld], row i at i - r0
   double* const gpart = GRID ? q.gpart + (long long)pb * n * C : nullptr;
   double* const gsum = GRID ? q.gsum + (long long)pb * n : nullptr;
@@ -353,8 +358,12 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
   unsigned* const gtop = cnt_top + QRG_LINE;
   __shared__ unsigned s_warp[QRC_MAXT / 32], s_top;   // largest high word of a warp's loads, of my rows (read by every CTA)
   bool live = true;                         // GRID: no wait of this thread has run out
-  if (!GRID) {
+  if (!GRID) {                              // what shared memory does not hold
     double* g = q.W + pb * q.wst + rank * (q.wst / C);
+    if (!mc_smem) {
+      mc = g;
+      g += qr_mc(k, C);
+    }
     if (!tri_smem) {
       tri = g;
       g += qr_tri(k);
@@ -605,6 +614,11 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
   } else {
     for (int c = tid >> 5; c < k; c += nt >> 5) {
       double* src = mc + (c / C) * k;
+      if (!mc_smem) {
+        const double* g = src + (c % C - rank) * (q.wst / C);
+        for (int i = lane; i <= c; i += 32) tri[c * (c + 1) / 2 + i] = __ldcg(g + i);
+        continue;
+      }
       if (C > 1) src = cluster.map_shared_rank(src, c % C);
       for (int i = lane; i <= c; i += 32) tri[c * (c + 1) / 2 + i] = src[i];
     }
@@ -1007,11 +1021,12 @@ namespace {
 constexpr size_t kQrSmemMax = 224 * 1024;
 
 int qr_ld(int m, int c) { return (((m + c - 1) / c) + 7) / 8 * 8 + 4; }   // = 4 mod 8: no bank conflicts
-size_t qr_head_bytes(int m, int n, int c) { return sizeof(double) * size_t(qr_head(n, std::min(m, n), c)); }
+size_t qr_head_bytes(int m, int n) { return sizeof(double) * size_t(qr_head(n, std::min(m, n))); }
+size_t qr_mc_bytes(int m, int n, int c) { return sizeof(double) * size_t(qr_mc(std::min(m, n), c)); }
 // Shared memory per CTA of an m x n factorisation with its rows split over c
-// CTAs and kept there (the triangle too where that still fits).
+// CTAs and kept there (the columns of M and the triangle too where they still fit).
 size_t qr_smem(int m, int n, int c) {
-  return qr_head_bytes(m, n, c) + sizeof(double) * size_t(qr_ld(m, c)) * size_t(n);
+  return qr_head_bytes(m, n) + sizeof(double) * size_t(qr_ld(m, c)) * size_t(n);
 }
 // One warp per SM quarter at least; four threads per column while that is no more than 512.
 int qr_threads(int n) { return std::max(128, std::min(QRC_MAXT, (4 * n + 31) / 32 * 32)); }
@@ -1049,9 +1064,10 @@ struct ClusterLaunch {
 double qr_clocks(int m, int n, int c, int np) {
   const double k = std::min(m, n), rows = std::ceil(double(m) / c);
   const double warps = qr_threads(n) / 32;
-  const size_t rows_b = qr_smem(m, n, c), all_b = rows_b + qr_tri_bytes(m, n);
+  const size_t rows_b = qr_smem(m, n, c), mc_b = rows_b + qr_mc_bytes(m, n, c), all_b = mc_b + qr_tri_bytes(m, n);
   const bool tri = all_b <= kQrSmemMax;
-  const int at_once = active_clusters(k_qr_cluster<false>, qr_threads(n), tri ? all_b : rows_b, c);
+  const int at_once = active_clusters(k_qr_cluster<false>, qr_threads(n),
+                                      tri ? all_b : mc_b <= kQrSmemMax ? mc_b : rows_b, c);
   if (at_once == 0) return 1e300;
   const double step = (c == 1 ? 3800.0 : 5600.0) + 180.0 * std::ceil(std::ceil(k / c) / warps);
   const double fp = 24.0 * rows * 2.0 * n / 32.0 * (n < 64 ? 1.3 : 1.0);
@@ -1093,7 +1109,7 @@ int qr_best_cluster(int m, int n, int np, int cmax, double* clocks) {
 // what is in shared memory, and how much of it.
 struct QrPlan {
   int C = 0;
-  bool w_smem = false, tri_smem = false;
+  bool w_smem = false, mc_smem = false, tri_smem = false;
   size_t bytes = 0;
 };
 
@@ -1117,20 +1133,28 @@ QrPlan qr_plan(int m, int n, int np, int qr_cmax) {
   QrPlan p;
   p.C = qr_best_cluster(m, n, np, lim, &clocks);
   p.w_smem = p.C > 0;
+  // (entries are indexed with 32 bits)
+  auto holds = [&](int c) { return qr_head_bytes(m, n) <= kQrSmemMax && (long long)qr_ld(m, c) * n < (1LL << 31); };
   if (!p.w_smem)
     for (int c = 1; c <= std::min(lim, std::max(1, m / 32)); c *= 2)
-      if (qr_head_bytes(m, n, c) <= kQrSmemMax) p.C = c;
+      if (holds(c)) p.C = c;
+  // rows, columns of M and triangle: each in shared memory where it still fits
   auto settle = [&] {
-    const size_t rows = p.w_smem ? qr_smem(m, n, p.C) : qr_head_bytes(m, n, p.C);
-    p.tri_smem = rows + qr_tri_bytes(m, n) <= kQrSmemMax;
-    p.bytes = rows + (p.tri_smem ? qr_tri_bytes(m, n) : 0);
+    auto add = [&](size_t b) {
+      const bool fits = p.bytes + b <= kQrSmemMax;
+      if (fits) p.bytes += b;
+      return fits;
+    };
+    p.bytes = p.w_smem ? qr_smem(m, n, p.C) : qr_head_bytes(m, n);
+    p.mc_smem = add(qr_mc_bytes(m, n, p.C));
+    p.tri_smem = add(qr_tri_bytes(m, n));
   };
   while (p.C > 0) {
     settle();
     if (active_clusters(k_qr_cluster<false>, qr_threads(n), p.bytes, p.C) > 0) break;
     p.C /= 2;   // clusters of this size cannot be launched here
     p.w_smem = p.C > 0 && qr_smem(m, n, p.C) <= kQrSmemMax;
-    if (p.C > 0 && qr_head_bytes(m, n, p.C) > kQrSmemMax) p.C = 0;
+    if (p.C > 0 && !holds(p.C)) p.C = 0;
   }
   std::lock_guard<std::mutex> g(mu);
   return cache.emplace(key, p).first->second;
@@ -1177,7 +1201,7 @@ TallPlan qr_grid(int m, int n, int np, double* clocks) {
   PEPS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int c = std::min(QRG_MAXP, sms / np);
   if (c < 2) return p;
-  const size_t b = qr_smem(m, n, c) + qr_tri_bytes(m, n);
+  const size_t b = qr_smem(m, n, c) + qr_mc_bytes(m, n, c) + qr_tri_bytes(m, n);
   if (b > kQrSmemMax || active_clusters(k_qr_cluster<true>, qr_threads(n), b, 1) < c * np) return p;
   const double rows = std::ceil(double(m) / c);
   *clocks = 14000.0 + n * (10500.0 + 24.0 * rows * 2.0 * n / 32.0 * (n < 64 ? 1.3 : 1.0));
@@ -1294,8 +1318,8 @@ void qr_whole(Ctx& cx, int m, int n, const TallPlan& p, const TP& A, long long r
   PEPS_CUDA(cudaMemsetAsync(a.gcount, 0, count * sizeof(double), cx.st));
   if (std::getenv("PEPS_VERBOSE")) std::fprintf(stderr, "[peps] qr %dx%d x%d: %d CTAs\n", m, n, np, p.P);
   Launch L(K_QR, cx.st, qr_flops(m, n) * np, 0);
-  int w_smem = 1, tri_smem = 1, ld = qr_ld(m, p.P), lanes = qr_lanes_log2(n);
-  void* args[] = {&a, &w_smem, &tri_smem, &ld, &lanes};
+  int w_smem = 1, mc_smem = 1, tri_smem = 1, ld = qr_ld(m, p.P), lanes = qr_lanes_log2(n);
+  void* args[] = {&a, &w_smem, &mc_smem, &tri_smem, &ld, &lanes};
   PEPS_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_qr_cluster<true>), dim3(p.P * np),
                                         dim3(qr_threads(n)), args, p.bytes, cx.st));
   PEPS_CHECK_LAUNCH();
@@ -1347,8 +1371,8 @@ void qr_direct(Ctx& cx, int m, int n, const TP& A, long long rs, long long cs, c
     a.wst = (long long)m * n;
     a.qst = (long long)m * k;
     a.tst = k;
-  } else if (!pl.w_smem || !pl.tri_smem) {
-    a.wst = C * ((pl.tri_smem ? 0 : tri) + (pl.w_smem ? 0 : (long long)ld * n));
+  } else if (!pl.w_smem || !pl.mc_smem || !pl.tri_smem) {
+    a.wst = C * ((pl.mc_smem ? 0 : qr_mc(k, C)) + (pl.tri_smem ? 0 : tri) + (pl.w_smem ? 0 : (long long)ld * n));
   }
   if (a.wst) {
     double* w = cx.scratch(size_t(np) * (a.wst + a.qst + a.tst) + 64);
@@ -1361,8 +1385,8 @@ void qr_direct(Ctx& cx, int m, int n, const TP& A, long long rs, long long cs, c
     k_qr_house<<<np, QR_THREADS, 0, cx.st>>>(a);
   } else {
     ClusterLaunch c(C * np, qr_threads(n), pl.bytes, C, cx.st);
-    PEPS_CUDA(cudaLaunchKernelEx(&c.cfg, k_qr_cluster<false>, a, pl.w_smem ? 1 : 0, pl.tri_smem ? 1 : 0, ld,
-                                 qr_lanes_log2(n)));
+    PEPS_CUDA(cudaLaunchKernelEx(&c.cfg, k_qr_cluster<false>, a, pl.w_smem ? 1 : 0, pl.mc_smem ? 1 : 0,
+                                 pl.tri_smem ? 1 : 0, ld, qr_lanes_log2(n)));
   }
   PEPS_CHECK_LAUNCH();
 }

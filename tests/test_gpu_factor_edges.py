@@ -46,3 +46,15 @@ def test_norm_with_tall_boundaries(peps, Ly, Lx, D, chi):
     A = synth.peps_gauss(Ly, Lx, 2, D, seed=60 + D)
     got, want = peps.norm(A, chi, mode="var", seed=2), O.norm(A, chi=chi, mode="var", seed=2)
     assert abs(got[0] - want[0]) < 1e-10 and got[1] == want[1]
+
+
+# Wide factorisations, through svd mode: rows of a square matrix in shared
+# memory and the triangular factor's columns beside them in global memory
+# (448 columns), everything but the sums in global memory (608 columns, where
+# those columns alone would fill the shared memory).
+@pytest.mark.parametrize("Ly,Lx,D,chi", [(4, 6, 4, 28), (4, 6, 4, 38)])
+def test_norm_with_wide_factorisations(peps, Ly, Lx, D, chi):
+    from paper_1311_6696_gb300 import synth
+    A = synth.peps_gauss(Ly, Lx, 2, D, seed=80 + D)
+    got, want = peps.norm(A, chi, mode="svd"), O.norm(A, chi=chi, mode="svd")
+    assert abs(got[0] - want[0]) < 1e-10 and got[1] == want[1]
