@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <set>
 #include <vector>
 
 #include "aux.cuh"
@@ -1034,11 +1035,18 @@ void cu0_launch(Ctx& cx, Cu0Lattice* lats, int nlat) {
     PEPS_CHECK_LAUNCH();
     return;
   }
-  static std::once_flag once;
-  std::call_once(once, [] {
-    PEPS_CUDA(cudaFuncSetAttribute(k_cu0_build, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCu0Smem)));
-    PEPS_CUDA(cudaFuncSetAttribute(k_cu0_als, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCu0Smem)));
-  });
+  {   // the kernels' shared memory is an attribute of the current device
+    static std::mutex mu;
+    static std::set<int> done;
+    int dev = 0;
+    PEPS_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> g(mu);
+    if (!done.count(dev)) {
+      PEPS_CUDA(cudaFuncSetAttribute(k_cu0_build, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCu0Smem)));
+      PEPS_CUDA(cudaFuncSetAttribute(k_cu0_als, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCu0Smem)));
+      done.insert(dev);
+    }
+  }
   const int T = tri_count(D);
   // Parts per site: about two CTAs per SM, no part without a no.
   const int parts = std::max(1, std::min(T, 2 * 152 / std::max(1, Lx * nlat)));
