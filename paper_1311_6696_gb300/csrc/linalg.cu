@@ -185,7 +185,7 @@ __device__ __forceinline__ double remote_sum(cg::cluster_group& cl, double* slot
 // of its SM quarter for 64 clocks whatever its active lanes, and a dependent
 // one waits as long (an addition after a shuffle 110), so a column step costs
 // its FP64 instructions: the fused update and inner products (2 per element),
-// a few sums, and the scalar chain (1 / norm and one reciprocal, ~900 clocks).
+// a few sums, and the scalar chain (1 / norm and one reciprocal, ~1,100 clocks).
 // Barriers cost ~50 clocks for a CTA, ~450 for a cluster, a remote load ~400.
 // Hence
 //   * one pass per column: the update with reflector j and the inner products
@@ -530,10 +530,7 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
       double y = 0.0, g = 0.0, h = 0.0;
       if (__double_as_longlong(s) << 1 != 0 && (__double2hiint(ss) >> 20 & 0x7ff) >= 23) {
         const double r = rsqrt(ss), e = fma(fabs(alpha), r, 1.0);
-        // 1 / e, e in [1, 2]: two Newton steps in one (cubic) from the FP32 value
-        const double z = double(__frcp_rn(float(e)));
-        const double d = fma(-e, z, 1.0);
-        g = r * r * fma(z, fma(d, d, d), z);
+        g = r * r * __drcp_rn(e);
         y = copysign(r, alpha);
         h = copysign(ss * r, alpha);
       }
@@ -715,13 +712,6 @@ __device__ __forceinline__ void jacobi_pair(int pr, int round, int qq, int& a, i
   }
 }
 
-// 1 / sqrt(x) for x in [1, 2]: one cubic step from the FP32 value.
-__device__ __forceinline__ double rsqrt_1to2(double x) {
-  const double y = double(rsqrtf(float(x)));
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
 // x * 2^k by the exponent bits; 0 below the normal range.
 __device__ __forceinline__ double scale2(double x, int k) {
   const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
@@ -874,7 +864,7 @@ __global__ void __launch_bounds__(SVC_MAXT) k_svd_cluster(const SvdArgs s, int h
             } else {
               t = ga / dl;   // far apart: the angle itself, beyond FP32's range
             }
-            const double w = fma(t, t, 1.0), c = rsqrt_1to2(w), ic = w * c;
+            const double w = fma(t, t, 1.0), c = rsqrt(w), ic = w * c;
             x = t * (db * es[a]);
             y = t * (da * es[b]);
             al[a] = fma(-t, ga, A2);
