@@ -1051,9 +1051,8 @@ Operand pack(Ctx& cx, const TP& src, int np, long long pad, int src_f64, const s
   const dim3 grid(unsigned(tiles), np);
   if (src_f64 == 0 && bf16 && !split && np == 1 && p.gr.n <= 1 && p.gk.n <= 1 && o.K % 4 == 0 &&
       (p.gk.n == 0 || p.gk.s[0] == 1) && (p.gr.n == 0 || p.gr.s[0] == o.K) &&
-      (reinterpret_cast<uintptr_t>(src.v(0)) & 15) == 0) {
+      (reinterpret_cast<uintptr_t>(src.v(0)) & 15) == 0 && o.rows * (o.K / 4) < (1LL << 31)) {   // 32-bit indices
     const long long quads = o.rows * (o.K / 4);
-    PEPS_REQUIRE(quads < (1LL << 31), "operand too large to pack");
     k_pack_rows<<<unsigned(std::min<long long>((quads + 255) / 256, 8 * 152)), 256, 0, cx.st>>>(
         static_cast<const float4*>(src.v(0)), quads, fast_divisor(o.K / 4), o.ld / 4, static_cast<uint2*>(o.hi));
   } else if (src_f64 == 2) {

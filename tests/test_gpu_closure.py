@@ -208,3 +208,23 @@ def test_gradient_at_widths_that_are_no_multiple_of_eight(env, W, n):
     assert abs(loss - want_loss) < 1e-2 * abs(want_loss)
     assert _rel(grad.cpu().double().numpy(), want.numpy()) < 1e-2
     assert np.max(np.abs(peps.mlp_predict(w, X.cuda(), 2, D, W).cpu().double().numpy() - sig.numpy())) < 1e-3
+
+
+def test_inference_on_more_than_two_to_the_33_inputs(env):
+    """Inputs beyond the row copy's 32-bit indices take the tiled operand pack.
+    The rows at the start, the middle and the end give the bits
+    of a batch of their own: the pack rounds every value alike, and both
+    batches have more tiles than SMs, so K is summed in one order."""
+    torch, peps = env
+    D, W = 8, 16
+    F = 2 * D ** 4 + 2 * D * D
+    n = 2 ** 33 // F + 700
+    if torch.cuda.mem_get_info()[0] < 60 << 30:
+        pytest.skip("needs 60 GB of device memory")
+    X = torch.empty(n, F, device="cuda").normal_(generator=torch.Generator(device="cuda").manual_seed(5))
+    X[:, F - D * D:] += 4.0 * torch.eye(D, device="cuda").reshape(-1)
+    w = peps.mlp_init(2, D, W, seed=9)
+    w[W * F + W + W * W + W:] = 0.05
+    got = peps.mlp_predict(w, X, 2, D, W)
+    for r in (0, n // 2, n - 20000):
+        assert torch.equal(got[r:r + 20000], peps.mlp_predict(w, X[r:r + 20000].clone(), 2, D, W))
