@@ -325,6 +325,17 @@ int peps_ipeps_cluster(const double* A, int d, int D, int on_device, const peps_
                        double* rho_h, double* rho_v, double* sigma, void* cuda_stream);
 
 /*
+ * peps_release_memory -- returns the library's unused memory on the current
+ *   device.  Workspaces come from a memory pool that keeps up to 4 GB mapped
+ *   between calls (mapping them anew takes most of a small call), and the rest
+ *   until the process next synchronises; an allocation of the library itself
+ *   that fails gives that memory back first, one by other code in the process
+ *   cannot.  Synchronises the device.  Env handles and
+ *   plans keep their memory.
+ */
+int peps_release_memory(void);
+
+/*
  * Failure detection (the paper has no counterpart).
  *
  * peps_set_iteration_caps -- caps of the library's iterations: the

@@ -1601,6 +1601,14 @@ int peps_ipeps_cluster(const double* A, int d, int D, int on_device, const peps_
   });
 }
 
+int peps_release_memory(void) {
+  return guard([&] {
+    require_device();
+    PEPS_CUDA(cudaDeviceSynchronize());   // frees still in a stream count once they have run
+    pool_trim();
+  });
+}
+
 int peps_set_iteration_caps(int cu0_half_sweeps, int jacobi_sweeps) {
   return guard([&] {
     PEPS_REQUIRE(cu0_half_sweeps >= 0 && cu0_half_sweeps <= 1000000 && jacobi_sweeps >= 0 &&

@@ -97,7 +97,7 @@ extern std::atomic<int> g_fault_alloc;      // > 0 while a PEPS_FAULT=alloc call
 // the stream is being captured the allocation becomes a memory node of the
 // graph.  Safe from several threads and streams, as cudaMallocAsync is.
 cudaError_t pool_alloc(void** p, size_t n, cudaStream_t st);
-// Returns the pool's kept memory to the device.
+// Returns the pool's kept memory to the device (peps_release_memory, and before an allocation fails).
 void pool_trim();
 
 // ---------------------------------------------------------------------------

@@ -32,7 +32,7 @@ EXPORTS = [
     "peps_plan_env", "peps_plan_launches", "peps_plan_free", "peps_plan_tune",
     "peps_set_iteration_caps", "peps_wait_selftest", "peps_boundary_fidelity", "peps_env_cluster_range",
     "peps_ipeps_cluster", "peps_bond_update", "peps_bond_update_cluster", "peps_mlp_train_state",
-    "peps_mlp_save", "peps_mlp_load", "peps_env_save", "peps_env_load",
+    "peps_mlp_save", "peps_mlp_load", "peps_env_save", "peps_env_load", "peps_release_memory",
 ]
 CLOSURE_WIDTH = 256
 
@@ -371,6 +371,12 @@ def cu0_noalloc(A_dev, sigma_dev, stream=None):
             raise ValueError(f"{name} is on cuda:{t.device.index}, the current device is "
                              f"cuda:{torch.cuda.current_device()}")
     _check(lib.peps_cu0_noalloc(A_dev.data_ptr(), Ly, Lx, d, D, sigma_dev.data_ptr(), _stream_ptr(stream)))
+
+
+def release_memory():
+    """Returns the memory that the library keeps between calls (up to 4 GB) to
+    the current device; env handles and plans keep theirs."""
+    _check(lib.peps_release_memory())
 
 
 def set_iteration_caps(cu0_half_sweeps: int = 0, jacobi_sweeps: int = 0):
