@@ -305,12 +305,16 @@ __device__ __forceinline__ unsigned load_acquire_gpu(const unsigned* p) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-// Bounded wait (about 2 s of SM clock) for `target` arrivals: false, with the
-// status word set, when it runs out.
-__device__ __forceinline__ bool wait_arrivals(const unsigned* p, unsigned target, int* flag) {
+// Bounded wait for `target` arrivals: false, with the status word set, when it
+// runs out.  About 2 s of SM clock between CTAs that are all running; the first
+// wait of a launch, which also waits for the SMs that other kernels on the
+// device still hold, gets a minute.
+constexpr long long QRG_WAIT = 4000000000LL, QRG_FIRST_WAIT = 120000000000LL;
+__device__ __forceinline__ bool wait_arrivals(const unsigned* p, unsigned target, int* flag,
+                                              long long limit = QRG_WAIT) {
   const long long start = clock64();
   while (int(load_acquire_gpu(p) - target) < 0) {
-    if (clock64() - start > 4000000000LL) {
+    if (clock64() - start > limit) {
       atomicOr(flag, FLAG_TIMEOUT);
       return false;
     }
@@ -402,7 +406,7 @@ __global__ void __launch_bounds__(QRC_MAXT) k_qr_cluster(const QrArgs q, int w_s
     if (tid == 0) {
       atomicMax(gtop, top);
       arrive_gpu(cnt_top);
-      live = wait_arrivals(cnt_top, unsigned(C), q.flag);
+      live = wait_arrivals(cnt_top, unsigned(C), q.flag, QRG_FIRST_WAIT);
       s_top = __ldcg(gtop);
     }
     __syncthreads();

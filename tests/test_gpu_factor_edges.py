@@ -58,3 +58,21 @@ def test_norm_with_wide_factorisations(peps, Ly, Lx, D, chi):
     A = synth.peps_gauss(Ly, Lx, 2, D, seed=80 + D)
     got, want = peps.norm(A, chi, mode="svd"), O.norm(A, chi=chi, mode="svd")
     assert abs(got[0] - want[0]) < 1e-10 and got[1] == want[1]
+
+
+def test_tall_boundaries_beside_other_work(peps):
+    """The CTAs of a QR on every SM wait for one another: with the device busy
+    on another stream when it is launched, the norm is the same to the bit."""
+    import torch
+    from paper_1311_6696_gb300 import synth
+    A = synth.peps_gauss(4, 6, 2, 5, seed=65)
+    alone = peps.norm(A, 60, mode="var", seed=2)
+    x = torch.randn(4096, 4096, device="cuda", dtype=torch.float64)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        for _ in range(8):
+            y = x @ x
+    assert peps.norm(A, 60, mode="var", seed=2) == alone
+    side.synchronize()
+    assert torch.equal(y, x @ x)
