@@ -1049,7 +1049,7 @@ void cu0_launch(Ctx& cx, Cu0Lattice* lats, int nlat) {
   }
   const int T = tri_count(D);
   // Parts per site: about two CTAs per SM, no part without a no.
-  const int parts = std::max(1, std::min(T, 2 * 152 / std::max(1, Lx * nlat)));
+  const int parts = std::max(1, std::min(T, 2 * num_sms() / std::max(1, Lx * nlat)));
   // Up to T = 10 (D = 4) a row's products take one SM about as long as the
   // exchange between several.
   const int C = T <= 10 ? 1 : 8;

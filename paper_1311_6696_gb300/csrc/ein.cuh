@@ -114,6 +114,9 @@ Dims ein_dims(const char* spec, const Dims& ad, const Dims& bd);
 void ein(Ctx& cx, const char* spec, const TP& A, const Dims& ad, const TP& B,
          const Dims& bd, const TP& C, double alpha = 1.0, double beta = 0.0);
 
+// SMs of the current device.
+int num_sms();
+
 // C = alpha * contract(A, B) on the tensor cores (tcgen05): operands are
 // FP64 (x_f64 = 1), FP32 or BF16 (x_f64 = 2) tensors, repacked to TF32 / BF16; C is written as
 // FP64 or FP32 in any index order; with Clo (FP32 output only) C receives the

@@ -5,8 +5,9 @@
 // its tile into element offsets once, keeps them in shared memory and
 // gathers the operands through them.
 //
-// What bounds it: the FP64 pipe issues 1.7 FMA per clock and SM (1.06 TFLOP/s
-// for the chip), so slow that a tile of any size keeps it busy -- a 16x16 tile
+// What bounds it: the FP64 pipe takes at most 2 FMA per clock and SM (one warp
+// instruction in 64 clocks and SM quarter; 1.26 TFLOP/s for the chip at 2070
+// MHz, of which torch's DGEMM of 8192^3 reaches 1.10), so slow that a tile of any size keeps it busy -- a 16x16 tile
 // needs 2 loaded doubles per 16 FMA -- and what decides the time is that every
 // SM gets the same share of the multiply-adds.  A contraction of 1M FMA on
 // 64x64 tiles occupies 16 SMs for 20 us; on 16x16 tiles, K split over a
@@ -20,11 +21,12 @@
 // Measured (us; before: 64x64-output tiles, split K with a second kernel):
 // 64x64 outputs, K 64 24.7 -> 6; 1024 outputs, K 64 78 -> 6.3; 256x256, K 16
 // 24.7 -> 6.3; 256x16, K 256 85 -> 10; 512x512, K 32 43 -> 23; 147456 outputs,
-// K 2304 801 -> 590 (1.15 TFLOP/s, the pipe's rate).
+// K 2304 801 -> 590 (1.15 TFLOP/s).
 // Independent problems of one shape (TP pointer sets) share a launch.
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <map>
 
@@ -328,18 +330,18 @@ std::vector<long long> strides_of(const Dims& d) {
   return s;
 }
 
+}  // namespace
+
 int num_sms() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 148;
-  }
+  static std::atomic<int> known[64];
+  int dev = 0, n = 0;
+  PEPS_CUDA(cudaGetDevice(&dev));
+  if (dev < 64) n = known[dev].load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  PEPS_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+  if (dev < 64) known[dev].store(n, std::memory_order_relaxed);
   return n;
 }
-
-}  // namespace
 
 Dims ein_dims(const char* spec, const Dims& ad, const Dims& bd) {
   Parsed p = parse(spec);
@@ -492,11 +494,11 @@ void ein(Ctx& cx, const char* spec, const TP& A, const Dims& ad, const TP& B,
     return;
   }
   // Tile and cluster: the least estimated time.  The FP64 pipe of an SM takes
-  // its CTAs' padded multiply-adds at 1.7 per clock whatever the tile (64x64,
-  // 64x32 and 64x16 measured no better than these two); a launch, its index
-  // set-up and first loads cost ~4,000 clocks, a CTA's own ~300, a further k
-  // tile a load latency that co-resident CTAs hide, and a cluster's exchange
-  // ~2,000, likewise.
+  // its CTAs' padded multiply-adds at 1.7 per clock on average, of the 2 it
+  // could, whatever the tile (64x64, 64x32 and 64x16 measured no better than
+  // these two); a launch, its index set-up and first loads cost ~4,000 clocks,
+  // a CTA's own ~300, a further k tile a load latency that co-resident CTAs
+  // hide, and a cluster's exchange ~2,000, likewise.
   struct Shape {
     int bm, bn, bk, nt;
   };

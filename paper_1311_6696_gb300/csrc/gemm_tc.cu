@@ -1042,7 +1042,7 @@ Operand pack(Ctx& cx, const TP& src, int np, long long pad, int src_f64, const s
   };
   p.rows_fast = inner(p.gr) < inner(p.gk) ? 1 : 0;
   auto tiles_of = [&](long long t) { return ((o.rows + t - 1) / t) * ((o.K + t - 1) / t); };
-  const bool small = tiles_of(64) * np < 152;
+  const bool small = tiles_of(64) * np < num_sms();
   const long long tiles = tiles_of(small ? 32 : 64);
   PEPS_REQUIRE(tiles < (1LL << 31), "operand too large to pack");
   const double moved = double(np) * double(o.rows) * double(o.K) *
@@ -1053,7 +1053,7 @@ Operand pack(Ctx& cx, const TP& src, int np, long long pad, int src_f64, const s
       (p.gk.n == 0 || p.gk.s[0] == 1) && (p.gr.n == 0 || p.gr.s[0] == o.K) &&
       (reinterpret_cast<uintptr_t>(src.v(0)) & 15) == 0 && o.rows * (o.K / 4) < (1LL << 31)) {   // 32-bit indices
     const long long quads = o.rows * (o.K / 4);
-    k_pack_rows<<<unsigned(std::min<long long>((quads + 255) / 256, 8 * 152)), 256, 0, cx.st>>>(
+    k_pack_rows<<<unsigned(std::min<long long>((quads + 255) / 256, 8 * num_sms())), 256, 0, cx.st>>>(
         static_cast<const float4*>(src.v(0)), quads, fast_divisor(o.K / 4), o.ld / 4, static_cast<uint2*>(o.hi));
   } else if (src_f64 == 2) {
     if (small)
@@ -1278,8 +1278,9 @@ void ein_tc(Ctx& cx, const char* spec, const TP& A, int a_f64, const Dims& ad, c
   g.kt_per = g.ktiles;
   const bool extras = chain && (chain->bias || chain->relu || chain->mask);
   g.parts = 1;
-  if (tiles < 152 && g.ktiles >= 4) {
-    const long long want = std::min<long long>((2 * 152 + tiles - 1) / tiles, g.ktiles / 2);
+  const int sms = num_sms();
+  if (tiles < sms && g.ktiles >= 4) {
+    const long long want = std::min<long long>((2 * sms + tiles - 1) / tiles, g.ktiles / 2);
     if (want > 1) {
       g.kt_per = int((g.ktiles + want - 1) / want);
       g.splitk = int((g.ktiles + g.kt_per - 1) / g.kt_per);

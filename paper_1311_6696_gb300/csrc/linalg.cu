@@ -1041,7 +1041,8 @@ struct ClusterLaunch {
 };
 
 // Estimated clocks of np factorisations on clusters of c CTAs, fitted to
-// measured times of shapes from 16x16 to 2304x64 on 1 to 16 CTAs (within 20%):
+// measured times of shapes from 16x16 to 2304x64 on 1 to 16 CTAs (within 20%;
+// 180x180 to 676x338 on 16 come out so as well):
 // a column costs its barriers, sums and scalars, its share of the back
 // substitutions, and the FP64 pipe 24 clocks per warp instruction and SM (19
 // at best), two per row and column; the pass leaves a quarter of that idle
@@ -1059,7 +1060,7 @@ double qr_clocks(int m, int n, int c, int np) {
   const double step = (c == 1 ? 3800.0 : 5600.0) + 180.0 * std::ceil(std::ceil(k / c) / warps);
   const double fp = 24.0 * rows * 2.0 * n / 32.0 * (n < 64 ? 1.3 : 1.0);
   const double waves = std::ceil(double(np) / at_once);
-  const double per_sm = std::ceil(std::min<double>(np, at_once) * c / 148.0);
+  const double per_sm = std::ceil(std::min<double>(np, at_once) * c / num_sms());
   return 10000.0 + waves * k * (step + per_sm * fp) * (tri ? 1.0 : 1.2);
 }
 
@@ -1159,7 +1160,7 @@ int tsqr_leaves(int m, int n, int np, double* clocks) {
     if (ml < n || ml < 16 * 32) break;
     double t1, t2;
     if (!qr_best_cluster(ml, n, np * L, 16, &t1) || !qr_best_cluster(L * n, n, np, 16, &t2)) continue;
-    const double t = t1 + t2 + 2.0 * double(np) * m * n * n / 148.0 / 3.0 + 20000.0;   // + the Q combine
+    const double t = t1 + t2 + 2.0 * double(np) * m * n * n / num_sms() / 3.0 + 20000.0;   // + the Q combine
     if (t < *clocks) {
       *clocks = t;
       best = L;
@@ -1183,10 +1184,7 @@ struct TallPlan {
 TallPlan qr_grid(int m, int n, int np, double* clocks) {
   TallPlan p;
   *clocks = 1e300;
-  int dev = 0, sms = 0;
-  PEPS_CUDA(cudaGetDevice(&dev));
-  PEPS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int c = std::min(QRG_MAXP, sms / np);
+  const int c = std::min(QRG_MAXP, num_sms() / np);
   if (c < 2) return p;
   const size_t b = qr_smem(m, n, c) + qr_mc_bytes(m, n, c) + qr_tri_bytes(m, n);
   if (b > kQrSmemMax || active_clusters(k_qr_cluster<true>, qr_threads(n), b, 1) < c * np) return p;
@@ -1409,7 +1407,7 @@ void svd_jacobi(Ctx& cx, int p, int q, const TP& A, long long rs, long long cs, 
     if (c > 1 && s.p / c < 2) break;
     const int at_once = active_clusters(k_svd_cluster, nt, smem, c);
     if (at_once == 0) continue;
-    const double per_sm = std::max(1.0, double(std::min(np, at_once)) * c / 148.0);
+    const double per_sm = std::max(1.0, double(std::min(np, at_once)) * c / num_sms());
     const double round = (c == 1 ? 2400.0 : 3600.0 + 70.0 * c) +
                          per_sm * (fits ? 1.0 : 2.0) * npair * (3.0 * s.p + 2.0 * s.q) / (1.4 * c);
     const double t = std::ceil(double(np) / at_once) * round;
