@@ -82,6 +82,9 @@ def _peaks():
 # stands, keyed by (workload, class); an entry is dropped whenever its kernel changes.
 TRAFFIC = {
     # (workload, class): (dram read + write bytes per launch, source)
+    ("c4", "qr_f64"): (4.52e6, "ncu, mean of the two k_qr_cluster launches of an 8192x128 fit step on a lane "
+                               "(four leaves 8.46 MB, their stacked R 0.59 MB); "
+                               "profiles/k_qr_cluster_rows3_20x20_D8_chi128.md"),
 }
 
 # Dense FP64 and TF32 peaks: measured at start-up by _measure_peaks (torch

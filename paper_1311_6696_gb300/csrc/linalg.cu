@@ -206,12 +206,12 @@ __device__ __forceinline__ double remote_sum(cg::cluster_group& cl, double* slot
 //     one back substitution in one warp, the columns dealt to the CTAs; the
 //     product runs at the FP64 pipe's rate.  Against one barrier, one set of
 //     sums and one pass per reflector (256x16 70 us, 512x32 158, 1024x64 441,
-//     64x64 280) this takes 53, 131, 381 and 203 us.
+//     64x64 280) this takes 56, 136, 396 and 209 us.
 // Measured (us, one matrix, with Q; before: scaled reflectors, update and inner
 // products in two passes, sums by one thread per column, Q one reflector at a
-// time): 256x16 117 -> 53, 512x32 236 -> 131, 1024x64 608 -> 381, 2304x64
-// 824 -> 618, 1620x180 3637 -> 2861, 8192x128 (tall-skinny, four leaves)
-// 3847 -> 2853; 16 of 36x36 270 -> 123 (those ran in global memory, one CTA
+// time): 256x16 117 -> 56, 512x32 236 -> 136, 1024x64 608 -> 396, 2304x64
+// 824 -> 643, 1620x180 3637 -> 2897, 8192x128 (tall-skinny, four leaves)
+// 3847 -> 2845; 16 of 36x36 270 -> 125 (those ran in global memory, one CTA
 // each).  Orthogonality stays at 1e-15 to 7e-15; |A - QR| is 1 to 3 eps of a
 // column's norm.  Shared memory holds the sums (88 bytes a column, to 2600
 // columns), then the rows, M's columns and the triangle, each while it fits; the
@@ -228,9 +228,9 @@ __device__ __forceinline__ double remote_sum(cg::cluster_group& cl, double* slot
 // adds those of a column, and everyone reads the n sums.
 // That costs a column about 5000 clocks more than one cluster's barrier and
 // sums, so it pays where the rows of 16 CTAs cost more than that.
-// Measured (us, one cluster or leaves -> every SM): 2304x64 619 -> 381,
-// 1024x128 1127 -> 796, 4096x128 2069 -> 966, 8192x128 2801 -> 1246,
-// 1620x180 2863 -> 1300, 8192x64 861 -> 498, three of 4096x128 2781 -> 1539.
+// Measured (us, one cluster or leaves -> every SM): 2304x64 643 -> 384,
+// 1024x128 1155 -> 797, 4096x128 2110 -> 969, 8192x128 2845 -> 1250,
+// 1620x180 2897 -> 1305, 8192x64 886 -> 501, three of 4096x128 2825 -> 1549.
 // Clusters of 8, summed first within the cluster and then over 15 to 19 of
 // them: 423, 776, 1010, 1362, 1602, 625, 1547.
 // ---------------------------------------------------------------------------
