@@ -676,8 +676,8 @@ struct SvdArgs {
 //   * the angle's tangent t = g / (|d| + sqrt(d^2 + g^2)), d = beta - alpha and
 //     g = 2 gamma, from one reciprocal root and one reciprocal, and its cosine
 //     from another root (taken from FP32 values, t leaves 1e-7 of the inner
-//     product to the next sweep: 4% faster, and 30 times less orthogonal where
-//     the last sweep did not come, 5x40 3e-14 against 9e-16);
+//     product to the next sweep: 3 to 10% faster, and less orthogonal where no
+//     further sweep came, graded 5x40 3e-14 against 9e-16);
 //   * scaled rotations (fast Givens): columns are kept as G = G' diag(d), and
 //     a rotation is one FMA per element, g_a' -= t d_b / d_a g_b',
 //     g_b' += t d_a / d_b g_a' (old values), d *= c; d goes back into the
